@@ -233,6 +233,7 @@ __device__ __forceinline__ void dftR(V (&v)[R]) {
 template <int N, int E>
 struct Plan;
 template <> struct Plan<32, 8>   { static constexpr int R1 = 8,  RM = 0,  RL = 4; };
+template <> struct Plan<64, 4>   { static constexpr int R1 = 4,  RM = 4,  RL = 4; };
 template <> struct Plan<64, 8>   { static constexpr int R1 = 8,  RM = 0,  RL = 8; };
 template <> struct Plan<128, 16> { static constexpr int R1 = 16, RM = 0,  RL = 8; };
 template <> struct Plan<256, 16> { static constexpr int R1 = 16, RM = 0,  RL = 16; };

@@ -70,9 +70,71 @@ const pcs::KernelEntry* find_entry(int H, int W, int cluster_size, int kernel = 
     return nullptr;
 }
 
+// Attributes set and resident clusters counted once per (device, entry).
+cudaError_t prepared(const pcs::KernelEntry* e, int* mc, int* aux) {
+    struct Known {
+        int dev;
+        const pcs::KernelEntry* e;
+        int mc, aux;
+    };
+    static std::mutex mu;
+    static std::vector<Known> known;
+    int dev = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    std::lock_guard<std::mutex> lk(mu);
+    for (const Known& k : known)
+        if (k.dev == dev && k.e == e) {
+            *mc = k.mc;
+            *aux = k.aux;
+            return cudaSuccess;
+        }
+    if ((err = e->prepare(mc, aux)) != cudaSuccess) return err;
+    known.push_back({dev, e, *mc, *aux});
+    return cudaSuccess;
+}
+
 }  // namespace
 
 namespace pcs {
+
+// The cheapest of the size's entries with a measured time: us per iteration, times the rounds when
+// the slices outnumber the resident clusters (the balanced schedule makes fractions of a round
+// count).  Without one: the first entry that answers to the kernel option.
+const KernelEntry* default_entry(int H, int W, int kernel, int S, int* max_clusters, int* max_clusters_aux,
+                                 cudaError_t* err) {
+    *err = cudaSuccess;
+    const KernelEntry* first = find_entry(H, W, 0, kernel);
+    if (!first) return nullptr;
+    if (first->us <= 0.f) {
+        *err = prepared(first, max_clusters, max_clusters_aux);
+        return first;
+    }
+    int dev = 0, sms = 0;
+    if ((*err = cudaGetDevice(&dev)) != cudaSuccess ||
+        (*err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return first;
+    const KernelEntry* best = nullptr;
+    double best_cost = 0.0;
+    for (const auto& e : entries()) {
+        if (e.H != H || e.W != W || e.resident != first->resident || e.us <= 0.f) continue;
+        int mc = 0, aux = 0;
+        if ((*err = prepared(&e, &mc, &aux)) != cudaSuccess) return first;
+        mc = std::min(mc, sms / e.C);  // one CTA per SM
+        if (mc < 1) continue;
+        const double cost = e.us * std::max(1.0, (double)S / mc);
+        if (!best || cost < best_cost) {
+            best = &e;
+            best_cost = cost;
+            *max_clusters = mc;
+            *max_clusters_aux = aux;
+        }
+    }
+    if (best) return best;
+    *err = prepared(first, max_clusters, max_clusters_aux);
+    return first;
+}
+
 // error text for the other translation units of the library
 pcs_status set_last_error(pcs_status st, const char* msg) { return fail(st, "%s", msg); }
 }  // namespace pcs
@@ -154,6 +216,7 @@ struct pcs_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
     const pcs::KernelEntry* entry = nullptr;  // NULL for an any-size context
+    bool by_count = false;                    // no variant options: each call takes the entry for its slice count
     pcs::GenSolver* gen = nullptr;            // any-size context: row/column kernels (pd_generic.cu)
     int max_clusters = 0;
     int max_clusters_aux = 0;
@@ -189,6 +252,7 @@ struct pcs_ctx {
     cudaGraphExec_t graph_exec = nullptr;
     pcs::PDParams graph_prm{};
     int graph_ncl = 0;
+    const pcs::KernelEntry* graph_entry = nullptr;
     std::mutex mu;
 };
 
@@ -272,6 +336,15 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
         ctx->last_iters = n_iter;
         return PCS_OK;
     }
+    PCS_CUDA(cudaSetDevice(ctx->device), "cudaSetDevice");
+    const pcs::KernelEntry* use = entry ? entry : ctx->entry;
+    int ncl = ncl_override > 0 ? ncl_override : ctx->max_clusters;
+    if (!entry && ctx->by_count) {
+        cudaError_t e = cudaSuccess;
+        int aux = 0;
+        use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, S, &ncl, &aux, &e);
+        PCS_CUDA(e, "kernel attributes");
+    }
     pcs::PDParams prm;
     std::memset(&prm, 0, sizeof(prm));  // padding too: the graph cache compares whole structs
     prm.field = field;
@@ -294,14 +367,12 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
     prm.resume = resume;
     prm.tv_iso = ctx->opt.tv;
     prm.weight = weight;
-    int ncl = ncl_override > 0 ? ncl_override : ctx->max_clusters;
     if (ctx->opt.max_clusters > 0 && ctx->opt.max_clusters < ncl) ncl = ctx->opt.max_clusters;
     if (ncl > S) ncl = S;
     if (ncl < 1) ncl = 1;
-    PCS_CUDA(cudaSetDevice(ctx->device), "cudaSetDevice");
     // more slices than resident clusters: balance the iterations over the clusters (streaming
     // kernel, plain solves; the monitored path's active flags keep whole slices)
-    const bool balanced = !active && ncl < S && n_iter > 0 && (entry ? entry : ctx->entry)->launch_sched;
+    const bool balanced = !active && ncl < S && n_iter > 0 && use->launch_sched;
     if (balanced) {
         if (!ctx->sched) {
             const size_t nseg = (size_t)ctx->max_slices * 2 + 1;
@@ -337,13 +408,13 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
         return balanced ? e->launch_sched(prm, ncl, ctx->stream) : e->launch(prm, ncl, ctx->stream);
     };
     if (entry && entry != ctx->entry) {  // another variant of the same size (monitored solves)
-        PCS_CUDA(launch(entry), "launch of the primal-dual kernel");
+        PCS_CUDA(launch(use), "launch of the primal-dual kernel");
         ctx->last_iters = n_iter;
         return PCS_OK;
     }
     if (ctx->opt.use_graph) {
         // replay the captured graph when the arguments are those it was captured with
-        const bool same = ctx->graph_exec && ncl == ctx->graph_ncl &&
+        const bool same = ctx->graph_exec && ncl == ctx->graph_ncl && use == ctx->graph_entry &&
                           std::memcmp(&prm, &ctx->graph_prm, sizeof(prm)) == 0;
         if (!same) {
             if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
@@ -351,7 +422,7 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
             ctx->graph_exec = nullptr;
             ctx->graph = nullptr;
             PCS_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal), "graph capture begin");
-            cudaError_t le = launch(ctx->entry);
+            cudaError_t le = launch(use);
             cudaGraph_t g = nullptr;
             cudaError_t ce = cudaStreamEndCapture(ctx->stream, &g);
             if (le != cudaSuccess) {
@@ -363,10 +434,11 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
             PCS_CUDA(cudaGraphInstantiate(&ctx->graph_exec, g, 0), "graph instantiate");
             ctx->graph_prm = prm;
             ctx->graph_ncl = ncl;
+            ctx->graph_entry = use;
         }
         PCS_CUDA(cudaGraphLaunch(ctx->graph_exec, ctx->stream), "graph launch");
     } else {
-        PCS_CUDA(launch(ctx->entry), "launch of the primal-dual kernel");
+        PCS_CUDA(launch(use), "launch of the primal-dual kernel");
     }
     ctx->last_iters = n_iter;
     return PCS_OK;
@@ -399,7 +471,7 @@ namespace {
 pcs_status ensure_aux(pcs_ctx* c) {
     if (c->partials) return PCS_OK;
     const size_t n = slice_elems(c) * (size_t)c->max_slices;
-    PCS_CUDA(cudaMalloc(&c->partials, (size_t)c->max_slices * c->entry->C * pcs::kReportSums * sizeof(double)),
+    PCS_CUDA(cudaMalloc(&c->partials, (size_t)c->max_slices * c->entry->aux_C * pcs::kReportSums * sizeof(double)),
              "cudaMalloc partials");
     PCS_CUDA(cudaMalloc(&c->Ldev, (size_t)c->max_slices * sizeof(double)), "cudaMalloc L");
     PCS_CUDA(cudaMalloc(&c->xa, n * sizeof(float)), "cudaMalloc power-iteration buffer");
@@ -455,7 +527,7 @@ pcs_status ctx_report(pcs_ctx* c, const float* field, const unsigned char* mask,
     a.weight = weight;
     PCS_CUDA(cudaSetDevice(c->device), "cudaSetDevice");
     PCS_CUDA(c->entry->launch_report(a, aux_clusters(c, S), c->stream), "launch of the report kernel");
-    const int C = c->entry->C;
+    const int C = c->entry->aux_C;
     std::vector<double> h((size_t)S * C * kReportSums);
     PCS_CUDA(cudaMemcpyAsync(h.data(), c->partials, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
              "D2H partials");
@@ -554,7 +626,13 @@ pcs_status pcs_create(pcs_ctx** out, int H, int W, int max_slices, const pcs_opt
         *out = c;
         return PCS_OK;
     }
-    if ((e = entry->prepare(&c->max_clusters, &c->max_clusters_aux)) != cudaSuccess) return bail(cuda_fail(e, "kernel attributes"));
+    c->by_count = o.cluster_size == 0 && o.threads == 0 && o.tile == 0 && entry->us > 0.f;
+    if (c->by_count) {
+        c->entry = pcs::default_entry(H, W, o.kernel, max_slices, &c->max_clusters, &c->max_clusters_aux, &e);
+    } else {
+        e = prepared(entry, &c->max_clusters, &c->max_clusters_aux);
+    }
+    if (e != cudaSuccess) return bail(cuda_fail(e, "kernel attributes"));
     if (c->max_clusters < 1)
         return bail(fail(PCS_ECUDA, "kernel %dx%d/C=%d cannot be made resident", H, W, entry->C));
 
@@ -731,12 +809,14 @@ pcs_status pcs_solve_slices_monitored(pcs_ctx* ctx, const float* field, const un
     const pcs::KernelEntry* e = nullptr;
     int ncl = 0;
     if (!ctx->gen) {
-        e = ctx->entry->resident ? find_entry(ctx->H, ctx->W, 0, 1) : ctx->entry;
-        if (!e) return fail(PCS_EUNSUPPORTED, "no streaming kernel for %d x %d", ctx->H, ctx->W);
+        e = ctx->entry;
         ncl = ctx->max_clusters;
-        if (e != ctx->entry) {
+        if (ctx->by_count || ctx->entry->resident) {
             int aux = 0;
-            PCS_CUDA(e->prepare(&ncl, &aux), "kernel attributes");
+            cudaError_t ce = cudaSuccess;
+            e = pcs::default_entry(ctx->H, ctx->W, 1, S, &ncl, &aux, &ce);
+            if (!e) return fail(PCS_EUNSUPPORTED, "no streaming kernel for %d x %d", ctx->H, ctx->W);
+            PCS_CUDA(ce, "kernel attributes");
         }
     }
     if (!ctx->active) PCS_CUDA(cudaMalloc(&ctx->active, (size_t)ctx->max_slices * sizeof(int)), "cudaMalloc flags");
@@ -838,6 +918,12 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
     pcs_status st = PCS_OK;
     for (const auto& e : entries()) {
         if (e.H != c.H || e.W != c.W || t.n_candidates >= 8) continue;
+        bool seen = false;  // the same kernel under the other kernel option
+        for (const auto& f : entries()) {
+            if (&f == &e) break;
+            seen = seen || f.launch == e.launch;
+        }
+        if (seen) continue;
         pcs_options o = b->opt;
         o.cluster_size = e.C;
         o.kernel = e.resident ? 2 : 1;

@@ -88,8 +88,6 @@ struct DeviceSetup {
     float2* twid = nullptr;
     bool tables[kNumSizes][2] = {};   // (size, axis) region uploaded
     bool twiddles[kNumSizes] = {};    // size's twiddle region uploaded
-    const pcs::KernelEntry* prepared[16] = {};
-    int max_clusters[16] = {};
 };
 
 constexpr int kMaxDevices = 64;
@@ -102,18 +100,6 @@ pcs_status err(pcs_status st, const char* what, cudaError_t e) {
     return pcs::set_last_error(st, buf);
 }
 
-const pcs::KernelEntry* default_entry(int H, int W) {
-    const pcs::KernelEntry* (*fns[])(int*) = {pcs::entries_64,  pcs::entries_128, pcs::entries_192,
-                                               pcs::entries_256, pcs::entries_384, pcs::entries_512};
-    for (auto fn : fns) {
-        int n = 0;
-        const pcs::KernelEntry* e = fn(&n);
-        for (int k = 0; k < n; ++k)
-            if (e[k].H == H && e[k].W == W) return &e[k];
-    }
-    return nullptr;
-}
-
 }  // namespace
 
 extern "C" pcs_status pcs_solve_slices_noalloc(const float* field, const unsigned char* mask, int H, int W,
@@ -121,8 +107,9 @@ extern "C" pcs_status pcs_solve_slices_noalloc(const float* field, const unsigne
                                                float* chi_out, int b0_axis, void* cuda_stream) {
     PCS_TRACE("pcs_solve_slices_noalloc");
     if (S < 0 || n_iter < 0) return pcs::set_last_error(PCS_EINVAL, "pcs_solve_slices_noalloc: S and n_iter must be >= 0");
-    const pcs::KernelEntry* entry = default_entry(H, W);
-    if (!entry) return pcs::set_last_error(PCS_EUNSUPPORTED, "pcs_solve_slices_noalloc: unsupported slice size");
+    bool compiled = false;
+    for (int n : kSizes) compiled = compiled || (H == n && W == n);
+    if (!compiled) return pcs::set_last_error(PCS_EUNSUPPORTED, "pcs_solve_slices_noalloc: unsupported slice size");
     if ((size_t)S * (size_t)H * (size_t)W > kMaxVoxels) {
         char buf[200];
         snprintf(buf, sizeof(buf),
@@ -161,18 +148,9 @@ extern "C" pcs_status pcs_solve_slices_noalloc(const float* field, const unsigne
             return err(PCS_ECUDA, "cudaGetSymbolAddress(twid)", e);
         d.ready = true;
     }
-    int slot = -1;
-    for (int k = 0; k < 16; ++k)
-        if (d.prepared[k] == entry || d.prepared[k] == nullptr) {
-            slot = k;
-            break;
-        }
-    if (slot < 0) return pcs::set_last_error(PCS_EUNSUPPORTED, "pcs_solve_slices_noalloc: too many sizes");
-    if (d.prepared[slot] == nullptr) {
-        int a = 0;
-        if ((e = entry->prepare(&d.max_clusters[slot], &a)) != cudaSuccess) return err(PCS_ECUDA, "kernel attributes", e);
-        d.prepared[slot] = entry;
-    }
+    int ncl = 0, aux = 0;
+    const pcs::KernelEntry* entry = pcs::default_entry(H, W, 0, S, &ncl, &aux, &e);
+    if (e != cudaSuccess) return err(PCS_ECUDA, "kernel attributes", e);
     int k_size = -1;
     for (int k = 0; k < kNumSizes; ++k)
         if (kSizes[k] == H && H == W) k_size = k;
@@ -223,7 +201,6 @@ extern "C" pcs_status pcs_solve_slices_noalloc(const float* field, const unsigne
     prm.tau = (float)tau;
     prm.inv_den = (float)(1.0 / (1.0 + sigma / lambda));
     prm.inv_den_slice = nullptr;
-    int ncl = d.max_clusters[slot];
     if (ncl > S) ncl = S;
     if (ncl < 1) ncl = 1;
     if ((e = entry->launch(prm, ncl, stream)) != cudaSuccess) return err(PCS_ECUDA, "kernel launch", e);

@@ -2,18 +2,20 @@
 #include "pd_launch.cuh"
 
 namespace pcs {
+using Aux = Geo<256, 256, 4, 1, 512>;
 static const KernelEntry k_entries[] = {
-    // default: 4-CTA clusters, one 512-thread CTA per SM (more slices than its resident clusters
-    // run on the balanced schedule)
-    make_entry<Geo<256, 256, 4, 1, 512>>(),
+    // 23.1 us per iteration of up to 36 slices (35 for the half-spectrum kernel in the same geometry,
+    // Geo<256, 256, 4, 1, 512>); larger clusters for fewer slices: 17.7 us for up to 15, 13.6 us for up to 8
+    make_pair_entry<GeoPair<256, 4, 512, true>, Aux>(23.1f),
+    make_pair_entry<GeoPair<256, 8, 256, false>, Aux>(17.7f),
+    make_pair_entry<GeoPair<256, 16, 128, false>, Aux>(13.6f),
     make_entry<Geo<256, 256, 4, 2>>(),
     make_resident_entry<GeoRes<256, 256, 8>>(),
     make_entry<Geo<256, 256, 2, 1>>(),
-    make_entry<Geo<256, 256, 8, 2>>(),
     // eight elements per lane, 512-thread CTAs (more warps per SM)
     make_resident_entry<GeoRes<256, 256, 8, 512, 8, 8>>(),
-    // other FFT tile shapes of the default geometry (the autotuner's choice): rows with 8
-    // elements per lane (16 lanes per row, two row passes), or columns with 8 (32 lanes per column)
+    // other FFT tile shapes: rows with 8 elements per lane (16 lanes per row, two row passes), or
+    // columns with 8 (32 lanes per column)
     make_entry<Geo<256, 256, 4, 1, 512, 8, 16>>(),
     make_entry<Geo<256, 256, 4, 1, 512, 16, 8>>(),
 };

@@ -5,6 +5,7 @@
 
 #include "pd_aux.cuh"
 #include "pd_cluster.cuh"
+#include "pd_pair.cuh"
 #include "pd_resident.cuh"
 
 namespace pcs {
@@ -13,7 +14,7 @@ namespace pcs {
 // diagnostics / step-size companions.
 struct KernelEntry {
     int H, W, C;
-    int resident;  // 1: state held on chip (pd_resident_kernel); 0: state streamed (pd_cluster_kernel)
+    int resident;  // the option value it answers to: 1 resident, 0 streaming (weighted and resumed solves)
     size_t smem;
     int threads;
     int tile;      // FFT tile shape: 100 x (elements per lane of the row transforms) + those of the columns
@@ -23,8 +24,13 @@ struct KernelEntry {
     cudaError_t (*launch)(const PDParams& prm, int n_clusters, cudaStream_t stream);
     cudaError_t (*launch_report)(const AuxParams& prm, int n_clusters, cudaStream_t stream);
     cudaError_t (*launch_opnorm)(const AuxParams& prm, int n_clusters, cudaStream_t stream);
-    // the balanced-schedule instantiation of the iteration kernel (NULL for the resident kernel)
+    // the balanced-schedule instantiation of the iteration kernel (NULL for pd_resident_kernel)
     cudaError_t (*launch_sched)(const PDParams& prm, int n_clusters, cudaStream_t stream);
+    int aux_C;     // cluster size of the diagnostics and power iteration
+    // Measured us per iteration with at most one CTA per SM; the entries of a size that have it give
+    // bit-identical results, and contexts without variant options take the cheapest for the call's
+    // slice count (default_entry in pcs_api.cu).  0: only by option or autotuner.
+    float us;
 };
 
 template <class G>
@@ -105,7 +111,37 @@ template <class G>
 constexpr KernelEntry make_entry() {
     return KernelEntry{G::H,           G::W,           G::C,       0,
                        G::SMEM_BYTES,  G::NT,          100 * G::ER + G::EC, &prepare_all<G>,
-                       &launch_pd<G>,  &launch_report<G>, &launch_opnorm<G>, &launch_pd_sched<G>};
+                       &launch_pd<G>,  &launch_report<G>, &launch_opnorm<G>, &launch_pd_sched<G>, G::C, 0.f};
+}
+
+// One-transform-pair variant (pd_pair.cuh), state on chip: it serves both kernel options (RES is the
+// one this entry answers to).  The diagnostics and power iteration use the half-spectrum geometry G.
+template <class GP>
+cudaError_t launch_pair(const PDParams& prm, int n_clusters, cudaStream_t stream) {
+    return launch_cluster<GP>(pd_pair_kernel<GP>, prm, GP::SMEM_BYTES, n_clusters, stream);
+}
+template <class GP>
+cudaError_t launch_pair_sched(const PDParams& prm, int n_clusters, cudaStream_t stream) {
+    return launch_cluster<GP>(pd_pair_kernel<GP, true>, prm, GP::SMEM_BYTES, n_clusters, stream);
+}
+template <class GP, class G>
+cudaError_t prepare_pair(int* max_clusters, int* max_clusters_aux) {
+    int a = 0, b = 0, c = 0;
+    cudaError_t e;
+    if ((e = prepare_cluster<GP>(pd_pair_kernel<GP>, GP::SMEM_BYTES, max_clusters)) != cudaSuccess) return e;
+    if ((e = prepare_cluster<GP>(pd_pair_kernel<GP, true>, GP::SMEM_BYTES, &c)) != cudaSuccess) return e;
+    if (c < *max_clusters) *max_clusters = c;
+    if ((e = prepare_cluster<G>(aux_report_kernel<G>, aux_smem<G>(), &a)) != cudaSuccess) return e;
+    if ((e = prepare_cluster<G>(aux_opnorm_kernel<G>, aux_smem<G>(), &b)) != cudaSuccess) return e;
+    *max_clusters_aux = a < b ? a : b;
+    return cudaSuccess;
+}
+template <class GP, class G, int RES = 0>
+constexpr KernelEntry make_pair_entry(float us) {
+    static_assert(GP::H == G::H && GP::W == G::W, "same slices");
+    return KernelEntry{GP::H,           GP::W,          GP::C,       RES,
+                       GP::SMEM_BYTES,  GP::NT,         100 * GP::E + GP::E, &prepare_pair<GP, G>,
+                       &launch_pair<GP>, &launch_report<G>, &launch_opnorm<G>, &launch_pair_sched<GP>, G::C, us};
 }
 
 // Resident variant: the iteration kernel keeps the state on chip; the
@@ -130,7 +166,7 @@ constexpr KernelEntry make_resident_entry() {
     using G = typename GR::B;
     return KernelEntry{GR::H,           GR::W,          GR::C,       1,
                        GR::SMEM_BYTES,  GR::NT,         100 * GR::ER + GR::EC, &prepare_res<GR>,
-                       &launch_res<GR>, &launch_report<G>, &launch_opnorm<G>, nullptr};
+                       &launch_res<GR>, &launch_report<G>, &launch_opnorm<G>, nullptr, G::C, 0.f};
 }
 
 // FP64 variant (precision study): iteration kernel only.
@@ -161,5 +197,11 @@ const KernelEntry* entries_192(int* n);
 const KernelEntry* entries_256(int* n);
 const KernelEntry* entries_384(int* n);
 const KernelEntry* entries_512(int* n);
+
+// The entry a call without variant options runs for S slices (kernel: 0 the size's default, 1, 2 the
+// option), how many of its clusters are resident (one CTA per SM) and how many of the auxiliary
+// kernels'; sets the kernels' attributes on the current device (cached).  NULL: none compiled.
+const KernelEntry* default_entry(int H, int W, int kernel, int S, int* max_clusters, int* max_clusters_aux,
+                                 cudaError_t* err);
 
 }  // namespace pcs
