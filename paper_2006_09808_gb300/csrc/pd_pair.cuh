@@ -57,7 +57,7 @@ namespace pcs {
 // ------------------------------------------------------------------ geometry
 
 // N x N slices, clusters of C CTAs of NT threads (two rows per lane group).
-// TMEM: state in tensor memory (NT = 512 only), else in shared memory.
+// TMEM: state in tensor memory (CTAs that fill an SM), else in shared memory.
 template <int N_, int C_, int NT_, bool TMEM_, int E_ = 0>
 struct GeoPair {
     static constexpr int N = N_, H = N_, W = N_, C = C_, NT = NT_;
@@ -81,7 +81,11 @@ struct GeoPair {
     static constexpr size_t SMEM_BYTES = BASE_BYTES + (SLOT_GLOBAL ? 0 : SLOT_BYTES);
     static_assert(NG * 2 == R && NG == PC, "two rows and one column pair per lane group");
     static_assert(T >= 8 && T <= 32 && (T & (T - 1)) == 0 && E % 4 == 0, "lane groups");
-    static_assert(!TMEM || (NT == 512 && E <= 16), "tensor-memory state: one CTA per SM");
+    // p in global scratch (thread order) when four arrays exceed the tensor memory
+    static constexpr bool P_GLOBAL = TMEM && (NT / 128) * 8 * E > 512;
+    static constexpr int TM_WORDS = (P_GLOBAL ? 6 : 8) * E;  // tensor-memory words per thread
+    static_assert(!TMEM || (NT > 256 && (NT / 128) * TM_WORDS <= 512), "tensor-memory state: one CTA per SM");
+    static_assert(E <= 32, "mask bits");
     static_assert(SMEM_BYTES <= 232448, "shared memory");
     static constexpr int TMEM_COLS = 512;
 };
@@ -286,6 +290,21 @@ __device__ __forceinline__ void dftRp(C2 (&v)[R]) {
         v[1] = csub(t, v[1]);
     } else if constexpr (R == 4) {
         dft4p<INV>(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 6) {
+        // n = 3 n1 + n2, k = k1 + 2 k2 (dft_composite of fft_core.cuh)
+        C2 y[3][2];
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) {
+            y[n2][0] = cadd(v[n2], v[3 + n2]);
+            const C2 t = csub(v[n2], v[3 + n2]);
+            y[n2][1] = (n2 == 0) ? t : cmulc<INV>(t, cos24(4 * n2), -sin24(4 * n2));
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < 2; ++k1) {
+            dft3p<INV>(y[0][k1], y[1][k1], y[2][k1]);
+#pragma unroll
+            for (int k2 = 0; k2 < 3; ++k2) v[k1 + 2 * k2] = y[k2][k1];
+        }
     } else if constexpr (R == 8) {
         dft8p<INV>(v);
     } else if constexpr (R == 12) {
@@ -445,15 +464,30 @@ struct ChunkId {
 template <class G>
 struct StTmem {
     unsigned base;
+    float4* gp;  // P_GLOBAL: this thread's p chunks, [NCH][NT]
     __device__ __forceinline__ void init(unsigned taddr, float*) {
         const int warp = threadIdx.x >> 5;
-        base = taddr + ((unsigned)(warp & 3) << 21) + (unsigned)((warp >> 2) * (8 * G::E));
+        base = taddr + ((unsigned)(warp & 3) << 21) + (unsigned)((warp >> 2) * G::TM_WORDS);
     }
-    __device__ __forceinline__ unsigned addr(ChunkId c) const { return base + (unsigned)(2 * G::E * c.a + 4 * c.q); }
+    __device__ __forceinline__ unsigned addr(ChunkId c) const {
+        const int a = (G::P_GLOBAL && c.a > kP) ? c.a - 1 : c.a;
+        return base + (unsigned)(2 * G::E * a + 4 * c.q);
+    }
+    // the four arrays' chunk q, in the order q_x, q_y, chi, p
+    __device__ __forceinline__ void load_all(float4 (&v)[4], int q) const {
+        if constexpr (G::P_GLOBAL) {
+            v[3] = __ldcg(gp + q * G::NT);
+            float4 t[3];
+            load(t, {{kQx, q}, {kQy, q}, {kChi, q}});
+            v[0] = t[0], v[1] = t[1], v[2] = t[2];
+        } else {
+            load(v, {{kQx, q}, {kQy, q}, {kChi, q}, {kP, q}});
+        }
+    }
     template <int K>
     __device__ __forceinline__ void load(float4 (&v)[K], const ChunkId (&c)[K]) const {
         unsigned w[4 * K];
-        static_assert(K == 1 || K == 2 || K == 4, "compiled block sizes");
+        static_assert(K >= 1 && K <= 4, "compiled block sizes");
         if constexpr (K == 1) {
             asm volatile("{\n\t" PCS_TMEM_LD "{%0,%1,%2,%3}, [%4];\n\t" PCS_TMEM_WAIT "\n\t}"
                          : PCS_OUT4(0)
@@ -463,6 +497,11 @@ struct StTmem {
                          "\n\t}"
                          : PCS_OUT4(0), PCS_OUT4(1)
                          : "r"(addr(c[0])), "r"(addr(c[1])));
+        } else if constexpr (K == 3) {
+            asm volatile("{\n\t" PCS_TMEM_LD "{%0,%1,%2,%3}, [%12];\n\t" PCS_TMEM_LD "{%4,%5,%6,%7}, [%13];\n\t" PCS_TMEM_LD
+                         "{%8,%9,%10,%11}, [%14];\n\t" PCS_TMEM_WAIT "\n\t}"
+                         : PCS_OUT4(0), PCS_OUT4(1), PCS_OUT4(2)
+                         : "r"(addr(c[0])), "r"(addr(c[1])), "r"(addr(c[2])));
         } else {
             asm volatile("{\n\t" PCS_TMEM_LD "{%0,%1,%2,%3}, [%16];\n\t" PCS_TMEM_LD "{%4,%5,%6,%7}, [%17];\n\t" PCS_TMEM_LD
                          "{%8,%9,%10,%11}, [%18];\n\t" PCS_TMEM_LD "{%12,%13,%14,%15}, [%19];\n\t" PCS_TMEM_WAIT "\n\t}"
@@ -475,6 +514,10 @@ struct StTmem {
                                __uint_as_float(w[4 * k + 3]));
     }
     __device__ __forceinline__ void st(int a, int q, float4 v) const {
+        if (G::P_GLOBAL && a == kP) {
+            __stcg(gp + q * G::NT, v);
+            return;
+        }
         asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr({a, q})),
                      "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
                      "r"(__float_as_uint(v.w)));
@@ -485,8 +528,12 @@ struct StTmem {
 template <class G>
 struct StShared {
     float4* base;  // [4 arrays x NCH][NT]
+    float4* gp;    // unused
     __device__ __forceinline__ void init(unsigned, float* mem) {
         base = reinterpret_cast<float4*>(mem) + threadIdx.x;
+    }
+    __device__ __forceinline__ void load_all(float4 (&v)[4], int q) const {
+        load(v, {{kQx, q}, {kQy, q}, {kChi, q}, {kP, q}});
     }
     template <int K>
     __device__ __forceinline__ void load(float4 (&v)[K], const ChunkId (&c)[K]) const {
@@ -720,6 +767,20 @@ struct PairSlots {
     }
 };
 
+// p in thread order (P_GLOBAL) to its rows.
+template <class G>
+__device__ __forceinline__ void pair_save_p(const PairCtx<G>& cx, float* p) {
+#pragma unroll 1
+    for (int q = 0; q < G::NCH; ++q) {
+        const float4 v = __ldcg(cx.st.gp + q * G::NT);
+        float* o = p + G::T * 2 * q;
+        __stcg(o, v.x);
+        __stcg(o + G::N, v.y);
+        __stcg(o + G::T, v.z);
+        __stcg(o + G::T + G::N, v.w);
+    }
+}
+
 // Bit e of the mask as 0.0f or the value v.
 __device__ __forceinline__ float bit_sel(unsigned bits, int e, float v) { return ((bits >> e) & 1u) ? v : 0.0f; }
 
@@ -757,13 +818,16 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
     const bool cont = prm.resume || it_b > 0;
     const int count = it_e - it_b;
 
-    // ---- mask bits (row a at bit e, row b at bit 16 + e) and state
-    unsigned mbits = 0;
+    // ---- mask bits of rows a and b, and state
+    unsigned mbit_a = 0, mbit_b = 0;
 #pragma unroll 1
-    for (int t = 0; t < 2 * E; ++t) {
-        const int r = t / E, e = t % E;
-        if (__ldg(prm.mask + row0 + r * N + T * e)) mbits |= 1u << (r * 16 + e);
+    for (int e = 0; e < E; ++e) {
+        mbit_a |= (__ldg(prm.mask + row0 + T * e) ? 1u : 0u) << e;
+        mbit_b |= (__ldg(prm.mask + row0 + N + T * e) ? 1u : 0u) << e;
     }
+    if (E <= 16) mbit_a |= mbit_b << 16;  // one register for both
+    // P_GLOBAL: p in the threads' order in chi_out's rows of the CTA (chi is on chip until the end)
+    cx.st.gp = reinterpret_cast<float4*>(prm.chi + (size_t)s * (N * N) + (size_t)cx.crank * G::R * N) + threadIdx.x;
 #pragma unroll 1
     for (int a = 0; a < 4; ++a) {
         const float* src = (a == kChi ? prm.chibar : a == kP ? prm.p : a == kQx ? prm.qx : prm.qy) + row0;
@@ -805,6 +869,10 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
 #pragma unroll 1
         while (true) {
             const bool last = (n == count);
+            if (G::P_GLOBAL && last) {  // chi_out is about to be written
+                pair_save_p<G>(cx, prm.p + row0);
+                __syncthreads();
+            }
             C2 x[E];
             if (!skip) {
                 // ================= phase A: chi, chibar, p of both rows
@@ -824,15 +892,19 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                 fft_pair<N, T, true>(x, RowBuf{cx.rows + fresh(grp) * (8 * N)}, cx.stw, fresh(g));  // x = (s v, u)
                 {
                     const F2 m_tau(-tau, -tau), m_tau_s(-tau_s, -tau_s), inv(inv_den, inv_den);
-                    const unsigned mb = fresh(mbits);
+                    const unsigned ma = fresh(mbit_a), mb = (E <= 16) ? ma >> 16 : fresh(mbit_b);
                     const float4* fp = fresh(fpk);
                     float4 f0 = __ldcg(fp), f1 = __ldcg(fp + G::NT);  // two chunks ahead
+                    float2 u0{}, u1{};
+                    if (G::SLOT_GLOBAL) u0 = slot.ld_up(0), u1 = slot.ld_up(1);
                     float pla = 0.f, plb = 0.f;
 #pragma unroll
                     for (int q = 0; q < NCH; ++q) {
                         float4 v[4];
-                        cx.st.load(v, {{kQx, q}, {kQy, q}, {kChi, q}, {kP, q}});
-                        const float2 qu = slot.ld_up(q);  // q_y of the row above row a
+                        cx.st.load_all(v, q);
+                        const float2 qu = G::SLOT_GLOBAL ? u0 : slot.ld_up(q);  // q_y of the row above row a
+                        u0 = u1;
+                        if (G::SLOT_GLOBAL && q + 2 < NCH) u1 = slot.ld_up(q + 2);
                         const float4 f = f0;
                         f0 = f1;
                         if (q + 2 < NCH) f1 = __ldcg(fp + (q + 2) * G::NT);
@@ -853,7 +925,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                             const F2 d2 = (ql - F2(qxa, qxb)) + (F2(up, qya) - F2(qya, qyb));
                             cn[c] = fma2(m_tau, d2, fma2(m_tau_s, x[e].x, c0));
                             const F2 bar = (cn[c] + cn[c]) - c0;
-                            F2 sw(bit_sel(mb, e, sigma), bit_sel(mb, 16 + e, sigma));
+                            F2 sw(bit_sel(ma, e, sigma), bit_sel(mb, e, sigma));
                             if (prm.weight) {
                                 const float* w = prm.weight + row0 + T * e;
                                 sw = F2(sigma * __ldg(w), sigma * __ldg(w + N));
@@ -887,7 +959,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                 // ================= phase B: q of both rows; q_y of row b after the wait for chibar of
                 // the next group's row a (isotropic TV: the projection of row b too)
                 {
-                    const unsigned mb = fresh(mbits);
+                    const unsigned ma = fresh(mbit_a), mb = (E <= 16) ? ma >> 16 : fresh(mbit_b);
                     const int iso = prm.tv_iso;
                     // chibar of the pixel to the right, one element ahead
                     float na = __shfl_sync(gm, x[0].x.lo(), src_right), nb = __shfl_sync(gm, x[0].x.hi(), src_right);
@@ -910,7 +982,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                                 ra = (e + 1 < E) ? na : ca;
                                 rb = (e + 1 < E) ? nb : cb;
                             }
-                            const float sma = bit_sel(mb, e, sigma), smb = bit_sel(mb, 16 + e, sigma);
+                            const float sma = bit_sel(ma, e, sigma), smb = bit_sel(mb, e, sigma);
                             const F2 bx = fma2(F2(sma, smb), F2(ra, rb) - x[e].x, F2(c ? v[0].z : v[0].x, c ? v[0].w : v[0].y));
                             vx[2 * c] = bx.lo(), vx[2 * c + 1] = bx.hi();
                             vy[2 * c] = fmaf(sma, cb - ca, vy[2 * c]);
@@ -922,15 +994,20 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                     }
                     cx.st.wait_st();
                     cluster_wait<C>();  // every gather of this iteration is done, too
+                    float2 below[NCH];  // slots in global memory: all loads in flight at once
+                    if constexpr (G::SLOT_GLOBAL) {
+#pragma unroll
+                        for (int q = 0; q < NCH; ++q) below[q] = slot.ld_dn(q);
+                    }
 #pragma unroll
                     for (int q = 0; q < NCH; ++q) {
-                        const float2 dn = slot.ld_dn(q);
+                        const float2 dn = G::SLOT_GLOBAL ? below[q] : slot.ld_dn(q);
                         float4 v[2];
                         cx.st.load(v, {{kQx, q}, {kQy, q}});
                         const float cb0 = x[2 * q].x.hi(), cb1 = x[2 * q + 1].x.hi();
                         // below the last row the difference is zero (Neumann)
-                        v[1].y = fmaf(bit_sel(mb, 16 + 2 * q, sigma), (has_down ? dn.x : cb0) - cb0, v[1].y);
-                        v[1].w = fmaf(bit_sel(mb, 17 + 2 * q, sigma), (has_down ? dn.y : cb1) - cb1, v[1].w);
+                        v[1].y = fmaf(bit_sel(mb, 2 * q, sigma), (has_down ? dn.x : cb0) - cb0, v[1].y);
+                        v[1].w = fmaf(bit_sel(mb, 2 * q + 1, sigma), (has_down ? dn.y : cb1) - cb1, v[1].w);
                         tv_prox(v[0].y, v[1].y, iso);
                         tv_prox(v[0].w, v[1].w, iso);
                         if (iso) cx.st.st(kQx, q, v[0]);
@@ -944,12 +1021,12 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
             // ================= phase C: forward transform of s W p + i b
             {
                 const F2 m_2tau(-2.0f * tau, -2.0f * tau);
-                const unsigned mb = fresh(mbits);
+                const unsigned ma = fresh(mbit_a), mb = (E <= 16) ? ma >> 16 : fresh(mbit_b);
                 float pla = 0.f, plb = 0.f;
 #pragma unroll
                 for (int q = 0; q < NCH; ++q) {
                     float4 v[4];
-                    cx.st.load(v, {{kQx, q}, {kQy, q}, {kChi, q}, {kP, q}});
+                    cx.st.load_all(v, q);
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
                         const int e = 2 * q + c;
@@ -961,7 +1038,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                         plb = shb;
                         // row a's q_y from above follows after the wait
                         const F2 d2 = (ql - F2(qxa, qxb)) + (F2(0.f, qya) - F2(qya, qyb));
-                        F2 sw(bit_sel(mb, e, scale), bit_sel(mb, 16 + e, scale));
+                        F2 sw(bit_sel(ma, e, scale), bit_sel(mb, e, scale));
                         if (prm.weight) {
                             const float* w = prm.weight + row0 + T * e;
                             sw = F2(scale * __ldg(w), scale * __ldg(w + N));
@@ -972,9 +1049,14 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                 }
                 cluster_wait<C>();  // q_y of the row above row a
                 const float up2 = has_up ? -2.0f * tau : 0.f;
+                float2 above[NCH];
+                if constexpr (G::SLOT_GLOBAL) {
+#pragma unroll
+                    for (int q = 0; q < NCH; ++q) above[q] = slot.ld_up(q);
+                }
 #pragma unroll
                 for (int q = 0; q < NCH; ++q) {
-                    const float2 qu = slot.ld_up(q);
+                    const float2 qu = G::SLOT_GLOBAL ? above[q] : slot.ld_up(q);
                     x[2 * q].y = F2(fmaf(up2, qu.x, x[2 * q].y.lo()), x[2 * q].y.hi());
                     x[2 * q + 1].y = F2(fmaf(up2, qu.y, x[2 * q + 1].y.lo()), x[2 * q + 1].y.hi());
                 }
@@ -1003,6 +1085,10 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
         }
     } else {
         // no iterations: chi = 0 (the zero start)
+        if (G::P_GLOBAL) {
+            pair_save_p<G>(cx, prm.p + row0);
+            __syncthreads();
+        }
 #pragma unroll 1
         for (int t = 0; t < 2 * E; ++t) __stcg(prm.chi + row0 + (t / E) * N + T * (t % E), 0.f);
         cluster_barrier<C>();
@@ -1010,6 +1096,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
     // ---- the state, for diagnostics and continuations: chi_{N-1} (chibar scratch), p, q
 #pragma unroll 1
     for (int a = 0; a < 4; ++a) {
+        if (G::P_GLOBAL && a == kP) continue;  // saved before chi_out was written
         float* dst = (a == kChi ? prm.chibar : a == kP ? prm.p : a == kQx ? prm.qx : prm.qy) + row0;
 #pragma unroll 1
         for (int q = 0; q < NCH; ++q) {

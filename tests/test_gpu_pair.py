@@ -18,7 +18,7 @@ VARIANTS = [
     (128, 8, 128, 808, True), (128, 4, 256, 808, True), (128, 2, 512, 808, True), (128, 1, 512, 1616, False),
     (192, 3, 512, 1212, True), (192, 6, 256, 1212, True), (192, 12, 128, 1212, True),
     (256, 4, 512, 1616, True), (256, 8, 256, 1616, True), (256, 16, 128, 1616, True),
-    (512, 16, 512, 1616, True),
+    (384, 8, 384, 2424, True), (512, 16, 512, 1616, True),
 ]
 # N iterations of FP32 rounding: a few ulp (6e-8) of the result per iteration, most of it damped
 N_ITER, TOL = 12, 12 * 4 * 6e-8
@@ -62,7 +62,7 @@ def test_variant_against_oracle(H, C, threads, tile, family, tv, axis, weighted,
         assert np.array_equal(got, solve(field, mask, lam, N_ITER, w, **opts))
 
 
-@pytest.mark.parametrize("H,S", [(64, 160), (128, 80), (192, 52), (256, 40), (512, 10)])
+@pytest.mark.parametrize("H,S", [(64, 160), (128, 80), (192, 52), (256, 40), (384, 18), (512, 10)])
 def test_more_slices_than_clusters_equal_slices_alone(H, S):
     """The balanced schedule continues a split slice from its stored state: bit for bit the slice alone."""
     pb = phantoms.volume(H, H, 2, seed=9, lam=5e-4, n_iter=9)
