@@ -26,26 +26,35 @@ constexpr int kGenMinLen = 8;
 constexpr int kGenMaxLen = 512;
 constexpr int kGenMaxRadix = 61;
 
-// Radices of n: factors 4 first, then 2, then the odd primes in increasing order.
+// Radices of n: the primes >= 5 first, the largest ahead (the first stage needs no twiddles, which
+// these apply in a pass of their own), then one 6 where 2 and 3 are left over, 4s, 2, 3s.
 bool gen_plan(int n, GenPlan* pl) {
     std::memset(pl, 0, sizeof(*pl));
     if (n < kGenMinLen || n > kGenMaxLen) return false;
     pl->n = n;
-    int m = n;
+    int m = n, twos = 0, threes = 0;
     auto push = [&](int r) {
         if (pl->nst >= pcs::kGenMaxStages) return false;
         pl->r[pl->nst++] = r;
-        m /= r;
         return true;
     };
-    while (m % 4 == 0)
-        if (!push(4)) return false;
-    while (m % 2 == 0)
-        if (!push(2)) return false;
-    for (int p = 3; p <= kGenMaxRadix && m > 1; p += 2)
-        while (m % p == 0)
+    for (; m % 2 == 0; m /= 2) ++twos;
+    for (; m % 3 == 0; m /= 3) ++threes;
+    for (int p = kGenMaxRadix; p >= 5 && m > 1; p -= 2)
+        for (bool prime = p % 3 != 0 && (p == 5 || p % 5 != 0) && (p == 7 || p % 7 != 0); prime && m % p == 0; m /= p)
             if (!push(p)) return false;
-    return m == 1;
+    if (m != 1) return false;
+    if (twos % 2 == 1 && threes > 0) {
+        if (!push(6)) return false;
+        --twos;
+        --threes;
+    }
+    for (; twos >= 2; twos -= 2)
+        if (!push(4)) return false;
+    if (twos && !push(2)) return false;
+    for (; threes > 0; --threes)
+        if (!push(3)) return false;
+    return true;
 }
 
 pcs_status failg(pcs_status st, const char* what, cudaError_t e = cudaSuccess) {
@@ -161,7 +170,9 @@ cudaError_t gen_create(GenSolver** out, int H, int W, int max_slices, int b0_axi
             cudaSuccess ||
         (e = cudaMemcpy(gs->tabs, tw_r.data(), W * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemcpy(gs->tabs + W, tw_c.data(), H * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(gen_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
+        (e = cudaFuncSetAttribute(gen_rows_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
+            cudaSuccess ||
+        (e = cudaFuncSetAttribute(gen_rows_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
             cudaSuccess ||
         (e = cudaFuncSetAttribute(gen_report_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
             cudaSuccess ||
@@ -238,15 +249,23 @@ cudaError_t gen_enqueue(GenSolver* gs, const float* field, const unsigned char* 
     // that grid (37.8 against 42.6 ms per 256x258x25 solve).  The first launch follows the
     // caller's own stream work and is serialised.
     const dim3 blk_r(kGenRowWarps * 32), blk_c(gs->col_threads);
+    // two warps per row pair (200 iterations, one / two warps, ms): 12 slices of 128x132 5.82 / 5.30, 9 of
+    // 90x170 9.07 / 7.33, 25 of 256x258 14.2 / 13.4; but 42 of 128x132 7.55 / 9.01: not for short rows
+    // that already fill the GPU (three 8-warp CTAs on each of 152 SMs)
+    const bool two = g.W >= 192 || 2 * pairs <= 152 * 3 * kGenRowWarps;
+    auto rows = two ? &gen_rows_kernel<64> : &gen_rows_kernel<32>;
+    const int per_cta = kGenRowWarps / (two ? 2 : 1);
+    const dim3 grid_l((pairs + per_cta - 1) / per_cta);
+    const size_t smem_l = sizeof(float2) * (size_t)g.W * (1 + 2 * per_cta);
     for (int it = 0; it < n_iter; ++it) {
         g.phase = 0;
         g.store = 1;
-        if ((e = launch_dep(gen_rows_kernel, grid_r, blk_r, gs->srows, st, it > 0, g)) != cudaSuccess ||
+        if ((e = launch_dep(rows, grid_l, blk_r, smem_l, st, it > 0, g)) != cudaSuccess ||
             (e = launch_dep(gs->cols_kern, grid_c, blk_c, gs->scols, st, true, g)) != cudaSuccess)
             return e;
         g.phase = 1;
         g.store = it + 1 < n_iter;
-        if ((e = launch_dep(gen_rows_kernel, grid_r, blk_r, gs->srows, st, true, g)) != cudaSuccess ||
+        if ((e = launch_dep(rows, grid_l, blk_r, smem_l, st, true, g)) != cudaSuccess ||
             (g.store && (e = launch_dep(gs->cols_kern, grid_c, blk_c, gs->scols, st, true, g)) != cudaSuccess))
             return e;
     }

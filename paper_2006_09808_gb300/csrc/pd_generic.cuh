@@ -68,15 +68,87 @@ __device__ __forceinline__ float2 gcmul(float2 a, float2 b) {
 // the runtime stage sizes.
 __device__ __forceinline__ int qdiv(int j, float inv) { return (int)(((float)j + 0.5f) * inv); }
 
-// Length pl.n DFT by one warp in shared memory (unnormalised; inv: exponent sign +).
+// Lanes that carry one transform together: a warp, or two warps of a CTA that synchronise on a named
+// barrier (id 1 + their number in the CTA).
+template <int LP>
+__device__ __forceinline__ void lanes_sync(int id) {
+    if constexpr (LP == 32) {
+        __syncwarp();
+    } else {
+        asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(LP) : "memory");
+    }
+}
+
+// (x, y) += (a, b) c, componentwise in one packed instruction.
+__device__ __forceinline__ void fma_pair(float2& acc, float2 v, float c) {
+    acc = __ffma2_rn(v, make_float2(c, c), acc);
+}
+
+// Direct part of a prime stage: outputs q' = qp and r - qp of NJ butterflies j = j0, j0 + dj, ...
+// (qp = 0: the plain sum), from the sums and differences sd[(q - 1) R + j] = (s_q, d_q) and v0[j]:
+// A = v_0 + sum s_q cos(2 pi m / r), B = sum d_q (-sin(2 pi m / r)), m = q qp mod r.  One coefficient
+// serves NJ butterflies, and the lanes that share them read the same (s, d): 2 NJ packed FMAs per
+// 1 + NJ loads (one lane per output and butterfly took 4 scalar FMAs per 3 loads).
+// A16: sd is 16-byte aligned.
+template <int NJ, bool A16>
+__device__ __forceinline__ void prime_outputs(const float2* sd, const float2* v0, float2* out, const float2* T, int r,
+                                              int R, int Ns, float invNs, int qp, int j0, int dj, float sg) {
+    float2 A[NJ], B[NJ];
+    int jj[NJ];
+#pragma unroll
+    for (int i = 0; i < NJ; ++i) {
+        jj[i] = min(j0 + i * dj, R - 1);  // past the end: repeats the last butterfly, stores nothing
+        A[i] = v0[jj[i]];
+        B[i] = make_float2(0.f, 0.f);
+    }
+    const int h = (r - 1) / 2;
+    int m = 0;
+#pragma unroll 2
+    for (int q = 1; q <= h; ++q) {
+        m += qp;
+        if (m >= r) m -= r;
+        const float2 c = T[m * R];  // (cos, -sin) of 2 pi m / r
+        const float2* row = sd + 2 * (q - 1) * R;
+#pragma unroll
+        for (int i = 0; i < NJ; ++i) {
+            float4 v;
+            if constexpr (A16) {
+                v = *reinterpret_cast<const float4*>(row + 2 * jj[i]);
+            } else {
+                const float2 sq = row[2 * jj[i]], dq = row[2 * jj[i] + 1];
+                v = make_float4(sq.x, sq.y, dq.x, dq.y);
+            }
+            fma_pair(A[i], make_float2(v.x, v.y), c.x);
+            fma_pair(B[i], make_float2(v.z, v.w), c.y);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NJ; ++i) {
+        const int j = j0 + i * dj;
+        if (j >= R) break;
+        const int k = j - qdiv(j, invNs) * Ns;
+        float2* o = out + (j - k) * r + k;
+        if (qp == 0) {
+            o[0] = A[i];
+        } else {
+            o[qp * Ns] = make_float2(A[i].x - sg * B[i].y, A[i].y + sg * B[i].x);
+            o[(r - qp) * Ns] = make_float2(A[i].x + sg * B[i].y, A[i].y - sg * B[i].x);
+        }
+    }
+}
+
+// Length pl.n DFT by LP lanes in shared memory (unnormalised; inv: exponent sign +).
 // Input in a, b is scratch; returns the buffer holding the result (which one depends
 // on the plan's radices).  Stage with
 // radix r after the radices so far multiply to Ns (R = n / r):
 //   X_out[(j / Ns) Ns r + k + q' Ns] = sum_q X_in[j + q R] w^(k q n/(Ns r)) w^(q q' R),
 // k = j mod Ns, w = exp(-+2 pi i / n), for j < R, q' < r.
-__device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan& pl, bool inv, int lane) {
+// A16: a and b are 16-byte aligned.
+template <int LP = 32, bool A16 = true>
+__device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan& pl, bool inv, int lane, int id = 0) {
     const int N = pl.n;
     const float sg = inv ? -1.f : 1.f;  // sign applied to the imaginary part of the forward twiddles
+    auto tw = [T, sg](int i) { return make_float2(T[i].x, sg * T[i].y); };
     int Ns = 1;
 #pragma unroll 1
     for (int st = 0; st < pl.nst; ++st) {
@@ -86,25 +158,19 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
         const float invNs = __frcp_rn((float)Ns), invR = __frcp_rn((float)R);
         if (r == 2) {
 #pragma unroll 1
-            for (int j = lane; j < R; j += 32) {
+            for (int j = lane; j < R; j += LP) {
                 const int k = j - qdiv(j, invNs) * Ns;
-                float2 t = T[k * step];
-                t.y *= sg;
-                const float2 v0 = a[j], v1 = gcmul(a[j + R], t);
+                const float2 v0 = a[j], v1 = gcmul(a[j + R], tw(k * step));
                 const int o = (j - k) * 2 + k;
                 b[o] = make_float2(v0.x + v1.x, v0.y + v1.y);
                 b[o + Ns] = make_float2(v0.x - v1.x, v0.y - v1.y);
             }
         } else if (r == 4) {
 #pragma unroll 1
-            for (int j = lane; j < R; j += 32) {
+            for (int j = lane; j < R; j += LP) {
                 const int k = j - qdiv(j, invNs) * Ns;
-                float2 t1 = T[k * step], t2 = T[2 * k * step], t3 = T[3 * k * step];
-                t1.y *= sg;
-                t2.y *= sg;
-                t3.y *= sg;
-                const float2 v0 = a[j], v1 = gcmul(a[j + R], t1), v2 = gcmul(a[j + 2 * R], t2),
-                             v3 = gcmul(a[j + 3 * R], t3);
+                const float2 v0 = a[j], v1 = gcmul(a[j + R], tw(k * step)), v2 = gcmul(a[j + 2 * R], tw(2 * k * step)),
+                             v3 = gcmul(a[j + 3 * R], tw(3 * k * step));
                 const float2 s02 = make_float2(v0.x + v2.x, v0.y + v2.y), d02 = make_float2(v0.x - v2.x, v0.y - v2.y);
                 const float2 s13 = make_float2(v1.x + v3.x, v1.y + v3.y), d13 = make_float2(v1.x - v3.x, v1.y - v3.y);
                 // -i d13 (forward) or +i d13 (inverse)
@@ -115,109 +181,98 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
                 b[o + 2 * Ns] = make_float2(s02.x - s13.x, s02.y - s13.y);
                 b[o + 3 * Ns] = make_float2(d02.x - rd.x, d02.y - rd.y);
             }
-        } else if (r == 3) {
+        } else if (r == 3 || r == 6) {
             const float h = 0.86602540378443865f;  // sin(2 pi / 3)
+            // one (r = 3) or two (r = 6) three-point transforms: q = 0, 2, 4 and q = 3, 5, 1 of the six
+            auto dft3 = [sg, h](float2& x, float2& y, float2& z) {
+                const float2 s = make_float2(y.x + z.x, y.y + z.y), d = make_float2(y.x - z.x, y.y - z.y);
+                const float2 m = make_float2(x.x - 0.5f * s.x, x.y - 0.5f * s.y);
+                const float2 rd = make_float2(sg * h * d.y, -sg * h * d.x);  // -i h d (forward) or +i h d (inverse)
+                x = make_float2(x.x + s.x, x.y + s.y);
+                y = make_float2(m.x + rd.x, m.y + rd.y);
+                z = make_float2(m.x - rd.x, m.y - rd.y);
+            };
+            if (r == 3) {
 #pragma unroll 1
-            for (int j = lane; j < R; j += 32) {
-                const int k = j - qdiv(j, invNs) * Ns;
-                float2 t1 = T[k * step], t2 = T[2 * k * step];
-                t1.y *= sg;
-                t2.y *= sg;
-                const float2 v0 = a[j], v1 = gcmul(a[j + R], t1), v2 = gcmul(a[j + 2 * R], t2);
-                const float2 s = make_float2(v1.x + v2.x, v1.y + v2.y), d = make_float2(v1.x - v2.x, v1.y - v2.y);
-                const float2 m = make_float2(v0.x - 0.5f * s.x, v0.y - 0.5f * s.y);
-                // -i h d (forward) or +i h d (inverse)
-                const float2 rd = make_float2(sg * h * d.y, -sg * h * d.x);
-                const int o = (j - k) * 3 + k;
-                b[o] = make_float2(v0.x + s.x, v0.y + s.y);
-                b[o + Ns] = make_float2(m.x + rd.x, m.y + rd.y);
-                b[o + 2 * Ns] = make_float2(m.x - rd.x, m.y - rd.y);
+                for (int j = lane; j < R; j += LP) {
+                    const int k = j - qdiv(j, invNs) * Ns;
+                    float2 v0 = a[j], v1 = gcmul(a[j + R], tw(k * step)), v2 = gcmul(a[j + 2 * R], tw(2 * k * step));
+                    dft3(v0, v1, v2);
+                    const int o = (j - k) * 3 + k;
+                    b[o] = v0;
+                    b[o + Ns] = v1;
+                    b[o + 2 * Ns] = v2;
+                }
+            } else {
+                // good-thomas: q = 3 n1 + 2 n2 (mod 6), q' = 3 k1 + 4 k2 (mod 6): no inner twiddles
+#pragma unroll 1
+                for (int j = lane; j < R; j += LP) {
+                    const int k = j - qdiv(j, invNs) * Ns;
+                    float2 v[6];
+                    v[0] = a[j];
+#pragma unroll
+                    for (int q = 1; q < 6; ++q) v[q] = gcmul(a[j + q * R], tw(q * k * step));
+                    dft3(v[0], v[2], v[4]);
+                    dft3(v[3], v[5], v[1]);
+                    const int o = (j - k) * 6 + k;
+                    auto put = [b, o, Ns](int qp, float2 x, float2 y, float sgn) {
+                        b[o + qp * Ns] = make_float2(x.x + sgn * y.x, x.y + sgn * y.y);
+                    };
+                    put(0, v[0], v[3], 1.f);
+                    put(3, v[0], v[3], -1.f);
+                    put(4, v[2], v[5], 1.f);
+                    put(1, v[2], v[5], -1.f);
+                    put(2, v[4], v[1], 1.f);
+                    put(5, v[4], v[1], -1.f);
+                }
             }
         } else {
-            // odd prime r >= 5: (1) pre-twiddle in place; (2) sums s_q = v_q + v_(r-q) and
-            // differences d_q = v_q - v_(r-q) into b; (3) outputs q' and r - q' together:
-            // A = v_0 + sum s_q cos(2 pi m / r), B = sum d_q (-sin(2 pi m / r)), m = q q' mod r,
-            // X_q' = A + i sg B, X_(r-q') = A - i sg B (forward sg = 1).  The result lands in a.
+            // odd prime r >= 5: (1) pre-twiddle in place (not in the first stage: k = 0); (2) sums
+            // s_q = v_q + v_(r-q) and differences d_q = v_q - v_(r-q) into b, side by side; (3) the
+            // outputs q' and r - q' together (prime_outputs).  The result lands in a.
+            if (Ns > 1) {
 #pragma unroll 1
-            for (int u = lane + R; u < N; u += 32) {
-                const int q = qdiv(u, invR), j = u - q * R;
-                float2 t = T[(j - qdiv(j, invNs) * Ns) * step * q];
-                t.y *= sg;
-                a[u] = gcmul(a[u], t);
+                for (int u = lane + R; u < N; u += LP) {
+                    const int q = qdiv(u, invR), j = u - q * R;
+                    a[u] = gcmul(a[u], tw((j - qdiv(j, invNs) * Ns) * step * q));
+                }
+                lanes_sync<LP>(id);
             }
-            __syncwarp();
             const int h = (r - 1) / 2;
+            float2 *sd = b, *v0 = b + 2 * h * R;
 #pragma unroll 1
-            for (int u = lane; u < R * (h + 1); u += 32) {
+            for (int u = lane; u < R * (h + 1); u += LP) {
                 const int q = qdiv(u, invR), j = u - q * R;
                 if (q == 0) {
-                    b[j] = a[j];
+                    v0[j] = a[j];
                 } else {
                     const float2 x = a[j + q * R], y = a[j + (r - q) * R];
-                    b[j + q * R] = make_float2(x.x + y.x, x.y + y.y);
-                    b[j + (r - q) * R] = make_float2(x.x - y.x, x.y - y.y);
+                    float2* o = sd + 2 * ((q - 1) * R + j);
+                    o[0] = make_float2(x.x + y.x, x.y + y.y);
+                    o[1] = make_float2(x.x - y.x, x.y - y.y);
                 }
             }
-            __syncwarp();
-            // q' = 0: X_0 = v_0 + sum s_q
+            lanes_sync<LP>(id);
+            // lanes: h + 1 outputs, as many groups of butterflies as fit (r <= 61: at least one)
+            const int nq = h + 1, jg = LP / nq, qp = lane % nq, g0 = lane / nq;
+            const int per = (R + jg - 1) / jg;  // butterflies per lane
+            if (g0 < jg) {
+                if (per <= 1) {
+                    prime_outputs<1, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, g0, jg, sg);
+                } else if (per == 2) {
+                    prime_outputs<2, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, g0, jg, sg);
+                } else if (per == 3) {
+                    prime_outputs<3, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, g0, jg, sg);
+                } else {
 #pragma unroll 1
-            for (int j = lane; j < R; j += 32) {
-                float2 acc = b[j];
-#pragma unroll 1
-                for (int q = 1; q <= h; ++q) {
-                    const float2 sq = b[j + q * R];
-                    acc.x += sq.x;
-                    acc.y += sq.y;
-                }
-                const int k = j - qdiv(j, invNs) * Ns;
-                a[(j - k) * r + k] = acc;
-            }
-            // q' = 1..h: two (j, q') units per lane at a time (independent chains)
-            const int NU = R * h;
-#pragma unroll 1
-            for (int u0 = lane; u0 < NU; u0 += 64) {
-                const bool has1 = (u0 + 32 < NU);
-                const int u1 = has1 ? u0 + 32 : u0;
-                const int t0 = qdiv(u0, invR), t1 = qdiv(u1, invR);
-                const int j0 = u0 - t0 * R, qp0 = 1 + t0;
-                const int j1 = u1 - t1 * R, qp1 = 1 + t1;
-                float2 A0 = b[j0], B0 = make_float2(0.f, 0.f);
-                float2 A1 = b[j1], B1 = make_float2(0.f, 0.f);
-                int m0 = 0, m1 = 0;
-#pragma unroll 1
-                for (int q = 1; q <= h; ++q) {
-                    m0 += qp0;
-                    if (m0 >= r) m0 -= r;
-                    m1 += qp1;
-                    if (m1 >= r) m1 -= r;
-                    const float2 c0 = T[m0 * R], c1 = T[m1 * R];  // (cos, -sin) of 2 pi m / r
-                    const float2 s0 = b[j0 + q * R], d0 = b[j0 + (r - q) * R];
-                    const float2 s1 = b[j1 + q * R], d1 = b[j1 + (r - q) * R];
-                    A0.x = fmaf(s0.x, c0.x, A0.x);
-                    A0.y = fmaf(s0.y, c0.x, A0.y);
-                    B0.x = fmaf(d0.x, c0.y, B0.x);
-                    B0.y = fmaf(d0.y, c0.y, B0.y);
-                    A1.x = fmaf(s1.x, c1.x, A1.x);
-                    A1.y = fmaf(s1.y, c1.x, A1.y);
-                    B1.x = fmaf(d1.x, c1.y, B1.x);
-                    B1.y = fmaf(d1.y, c1.y, B1.y);
-                }
-                const int k0 = j0 - qdiv(j0, invNs) * Ns;
-                const int ob0 = (j0 - k0) * r + k0;
-                a[ob0 + qp0 * Ns] = make_float2(A0.x - sg * B0.y, A0.y + sg * B0.x);
-                a[ob0 + (r - qp0) * Ns] = make_float2(A0.x + sg * B0.y, A0.y - sg * B0.x);
-                if (has1) {
-                    const int k1 = j1 - qdiv(j1, invNs) * Ns;
-                    const int ob1 = (j1 - k1) * r + k1;
-                    a[ob1 + qp1 * Ns] = make_float2(A1.x - sg * B1.y, A1.y + sg * B1.x);
-                    a[ob1 + (r - qp1) * Ns] = make_float2(A1.x + sg * B1.y, A1.y - sg * B1.x);
+                    for (int j = g0; j < R; j += 4 * jg) prime_outputs<4, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, j, jg, sg);
                 }
             }
-            __syncwarp();
+            lanes_sync<LP>(id);
             Ns *= r;
             continue;  // result in a: no swap
         }
-        __syncwarp();
+        lanes_sync<LP>(id);
         float2* t = a;
         a = b;
         b = t;
@@ -226,7 +281,11 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
     return a;
 }
 
-// Row kernel: a warp takes rows i0 = 2 pr, i1 = i0 + 1 of one slice.
+// Row kernel: LP lanes (one or two warps) take rows i0 = 2 pr, i1 = i0 + 1 of one slice.  The kernel is
+// bound by latency (25 slices of 256 x 258: half of the issue slots used by 21 warps per SM), which a
+// second warp per pair shortens; where the pairs fill the GPU with one warp each and the row is short,
+// the second only adds idle lanes (host rule in gen_enqueue).
+template <int LP>
 __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int H = g.H, W = g.W, M1 = g.M1;
@@ -234,10 +293,11 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
     for (int t = threadIdx.x; t < W; t += blockDim.x) T[t] = g.trow[t];
     __syncthreads();
     grid_dependency_wait();  // the previous launch's spectrum and state complete
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pair = blockIdx.x * kGenRowWarps + warp;
-    if (pair >= g.S * (H / 2)) return;  // whole warps; no CTA barrier below
-    float2* bufa = T + W + (size_t)warp * 2 * W;
+    constexpr int PAIRS = kGenRowWarps * 32 / LP;  // row pairs per CTA
+    const int lane = threadIdx.x % LP, wl = threadIdx.x & 31, grp = threadIdx.x / LP, bar = 1 + grp;
+    const int pair = blockIdx.x * PAIRS + grp;
+    if (pair >= g.S * (H / 2)) return;  // whole groups; no CTA barrier below
+    float2* bufa = T + W + (size_t)grp * 2 * W;
     float2* bufb = bufa + W;
     const int s = pair / (H / 2);
     if (g.active && !g.active[s]) return;  // frozen slice (monitored solves): state kept as is
@@ -248,7 +308,7 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
 
     // z = a + i b from the two half-spectrum rows (Hermitian extension beyond M1)
 #pragma unroll 3
-    for (int k = lane; k < W; k += 32) {
+    for (int k = lane; k < W; k += LP) {
         float2 z;
         if (k < M1) {
             const float2 A = __ldcg(sp0 + k), B = __ldcg(sp1 + k);
@@ -259,8 +319,8 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
         }
         bufa[k] = z;
     }
-    __syncwarp();
-    float2* u = warp_dft(bufa, bufb, T, g.prow, true, lane);
+    lanes_sync<LP>(bar);
+    float2* u = warp_dft<LP>(bufa, bufb, T, g.prow, true, lane, bar);
     float2* o = (u == bufa) ? bufb : bufa;
     const float sigma = g.sigma, tau = g.tau;
     // each element is read and written by one lane only: the state arrays do not alias
@@ -282,7 +342,7 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
         const bool down1 = (i1 + 1 < H);
         const float inv_den = g.inv_den_slice ? __ldg(g.inv_den_slice + s) : g.inv_den;
 #pragma unroll 2
-        for (int m0 = 0; m0 < NP; m0 += 32) {
+        for (int m0 = 0; m0 < NP; m0 += LP) {
             const int m = m0 + lane;
             const bool act = m < NP;
             const int n = 2 * (act ? m : NP - 1);  // inactive lanes shadow the last pair (no stores)
@@ -295,7 +355,7 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
             if (n + 2 >= W) {  // past the last column the difference is zero (Neumann)
                 c0r = c0.y;
                 c1r = c1.y;
-            } else if (lane == 31 || m + 1 >= NP) {
+            } else if (wl == 31 || m + 1 >= NP) {
                 c0r = __ldcg(cbar + a0 + 2);
                 c1r = __ldcg(cbar + a1 + 2);
             }
@@ -349,7 +409,7 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
         // q is zero wherever the 0/1 mask is (zero start, masked increments), so M q = q.
         const bool up0 = (i0 > 0), down1 = (i1 + 1 < H);
 #pragma unroll 2
-        for (int m0 = 0; m0 < NP; m0 += 32) {
+        for (int m0 = 0; m0 < NP; m0 += LP) {
             const int m = m0 + lane;
             const bool act = m < NP;
             const int n = 2 * (act ? m : NP - 1);
@@ -364,7 +424,7 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
             if (n == 0) {
                 qxl0 = 0.f;
                 qxl1 = 0.f;
-            } else if (lane == 0) {
+            } else if (wl == 0) {
                 qxl0 = __ldcg(qxp + a0 - 1);
                 qxl1 = __ldcg(qxp + a1 - 1);
             }
@@ -393,12 +453,12 @@ __global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g
             }
         }
     }
-    __syncwarp();
+    lanes_sync<LP>(bar);
     if (g.phase == 0 || g.store) {
-        float2* Z = warp_dft(o, u, T, g.prow, false, lane);
+        float2* Z = warp_dft<LP>(o, u, T, g.prow, false, lane, bar);
         // split: A = (Z(k) + conj Z(-k)) / 2, B = (Z(k) - conj Z(-k)) / (2 i)
 #pragma unroll 3
-        for (int k = lane; k < M1; k += 32) {
+        for (int k = lane; k < M1; k += LP) {
             const float2 zk = Z[k], zm = Z[k == 0 ? 0 : W - k];
             __stcg(sp0 + k, make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y)));
             __stcg(sp1 + k, make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x)));
@@ -683,7 +743,7 @@ __global__ void __launch_bounds__(kGenColTile * 32) gen_cols_kernel(GenParams g)
         const int kx = kx0 + warp;
         float2* a = cols + (size_t)warp * CS;
         float2* b = a + H;
-        float2* X = warp_dft(a, b, T, g.pcol, false, lane);
+        float2* X = warp_dft<32, false>(a, b, T, g.pcol, false, lane);
         const float fx = (float)kx / (float)W;
         const float scale = 1.0f / ((float)H * (float)W);
 #pragma unroll 1
@@ -696,7 +756,7 @@ __global__ void __launch_bounds__(kGenColTile * 32) gen_cols_kernel(GenParams g)
         }
         __syncwarp();
         // both directions swap the buffers equally often: the result is back in a
-        warp_dft(X, X == a ? b : a, T, g.pcol, true, lane);
+        warp_dft<32, false>(X, X == a ? b : a, T, g.pcol, true, lane);
     }
     __syncthreads();
     if (c < ncol) {
