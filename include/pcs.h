@@ -135,12 +135,14 @@ PCS_API pcs_status pcs_set_stream(pcs_ctx *ctx, void *cuda_stream);
  *   tau, sigma  primal and dual steps, > 0 (the paper uses tau = sigma = 1/||K||;
  *               see pcs_opnorm); tau*sigma*||K||^2 <= 1 is the caller's duty
  *   n_iter  >= 0 (0 gives chi = 0)
- *   chi_out device, [S][H][W] float32, caller-owned; also serves as the
- *           primal iterate during the solve (must not alias field)
+ *   chi_out device, [S][H][W] float32, caller-owned; also serves as scratch
+ *           during the solve (must not alias field)
  *   rep     NULL, or a host array of S reports; when given, the call also
  *           evaluates the FP64 diagnostics and synchronises the stream
  * All device pointers must be 16-byte aligned.  Slices are independent: the
- * result for a slice does not depend on the other slices in the call.
+ * result for a slice does not depend on the other slices in the call.  A
+ * context whose options leave cluster_size, threads and tile at 0 takes, for
+ * each call, the cluster size that suits S; those of a size give the same bits.
  * Errors: PCS_EINVAL, PCS_ECUDA.
  */
 PCS_API pcs_status pcs_solve_slices(pcs_ctx *ctx, const float *field, const unsigned char *mask, int S,
@@ -259,7 +261,7 @@ PCS_API pcs_status pcs_solve_slices_f64(const double *field, const unsigned char
  * s0, s1: device complex float32, interleaved (re, im), n_voxels each, 16-byte
  * aligned.  field_out, weight_out: device float32 [n_voxels], 8-byte aligned;
  * mask_out: device uint8 [n_voxels], 2-byte aligned.  Asynchronous on
- * cuda_stream (a small stream-ordered scratch allocation).  Errors: PCS_EINVAL (NULL, misaligned, t_shift or b0 <= 0,
+ * cuda_stream, without any allocation (field_out holds per-CTA maxima meanwhile).  Errors: PCS_EINVAL (NULL, misaligned, t_shift or b0 <= 0,
  * threshold < 0), PCS_ECUDA.  n_voxels = 0 is a no-op.
  */
 PCS_API pcs_status pcs_field_map(const float *s0, const float *s1, size_t n_voxels, double t_shift_s,
