@@ -39,11 +39,12 @@ WORKLOAD = "256x256x64 slices, 500 PD iterations, lambda=5e-4 (seeds/needles pha
 ALG_BYTES_PER_VOXEL_ITER = 37  # read+write chi, p, qx, qy (4 x 8 B) + read dB (4 B) + mask (1 B)
 ALG_FLOPS_PER_VOXEL_ITER = 10 * 16 + 30  # 2 real 2-D FFT round trips (10 log2(HW)) + pointwise/stencil
 L2_FLUSH_BYTES = 256 << 20
-# What ncu shows limiting the fused iteration kernel (profiles/pd_cluster_kernel_256x256x64.txt): the
-# slices in flight stay in L2, DRAM is nearly idle, and the row phases wait on L2 and distributed
-# shared-memory round trips; the HBM figure below is the useful-bytes roofline of the target.
-LIMITER_2D = "latency of L2 and DSMEM round trips (L2-resident working set; DRAM ~3% busy)"
-PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "pd_cluster_kernel_256x256x64.txt")
+# What ncu shows limiting the fused iteration kernel (profiles/pd_pair_kernel_256x256x64.txt): the
+# state stays on chip, DRAM and L2 are nearly idle; packed FP32 issue, the exchange through distributed
+# shared memory and the cluster barriers share the time.  The HBM figure below is the useful-bytes
+# roofline of the target.
+LIMITER_2D = "packed FP32 issue, DSMEM exchange and cluster barriers (state on chip; DRAM < 1% busy)"
+PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "pd_pair_kernel_256x256x64.txt")
 
 
 def dist_env():
@@ -59,7 +60,7 @@ def kernel_source_hash():
     taken from); the variant table and launch glue are host code."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2006_09808_gb300", "csrc")
-    for name in ("fft_core.cuh", "pd_cluster.cuh"):  # the iteration kernel's device code
+    for name in ("fft_core.cuh", "pd_cluster.cuh", "pd_pair.cuh"):  # the iteration kernel's device code
         for line in open(os.path.join(csrc, name), encoding="utf-8"):
             code = line.split("//", 1)[0].rstrip()
             if code:
@@ -489,7 +490,7 @@ def run_native(args):
                 "threads": args.threads or "default",
             },
             "roofline": {
-                "bound": "latency (L2/DSMEM)", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+                "bound": "latency (DSMEM, barriers) and FP32 issue", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": achieved / hbm_peak, "traffic": traffic,
                 "frac_of": "the measured HBM copy peak, in useful bytes (37 B per voxel-iteration)",
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else peak_kind,
@@ -955,7 +956,7 @@ def run_uneven(args):
                                    "{2e-4, 5e-4, 1e-3}, 400 PD iterations, one pcs_batch_solve per step",
                        "voxels": work // n_iter, "n_iter": n_iter,
                        "l2": "flushed between steps (256 MiB device write); inputs 1.3 GB > L2"},
-            "roofline": {"bound": "latency (L2/DSMEM)", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+            "roofline": {"bound": "latency (DSMEM, barriers) and FP32 issue", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "traffic": None,
                          "frac_of": "the measured HBM copy peak, in useful bytes (37 B per voxel-iteration)",
                          "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",

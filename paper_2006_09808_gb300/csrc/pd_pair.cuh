@@ -25,8 +25,8 @@
 //
 // A group of T lanes carries rows a = 2j, b = 2j + 1 of the slice for the whole solve, so every thread
 // owns the same 2E pixels throughout and their chi, p, qx, qy never leave the SM: in tensor memory
-// (StTmem: 512 threads x 8E words, 256 KB for E = 16; these CTAs fill the SM's registers, so no other
-// CTA competes for the allocation) or, for small CTAs, in shared memory (StShared).  Neighbouring
+// (StTmem: 512 threads x 8E words, 256 KB for E = 16; more than half of the SM's shared memory each,
+// so no two of these CTAs share an SM and the allocation never waits for a peer) or, for small CTAs, in shared memory (StShared).  Neighbouring
 // rows of other groups pass through one row slot per group boundary, which carries chibar of the
 // lower group's row a up and then q_y of the upper group's row b down.
 //
@@ -38,14 +38,13 @@
 // scatters both rows with one 16-byte access; the 16 lanes of a group cover whole 128-byte lines of
 // one CTA, and the strided accesses of the column pass spread over the banks.
 //
-// What bounds it (256 x 256, 4 CTAs of 512 threads, 36 slices): 64 x 500 iterations take 20.0 ms, 31.1
-// for pd_cluster.cuh's kernel in the same geometry, with 15% of the FP32 lanes busy in both.  On the
-// way there: scalar transforms of one row after the other, state in tensor memory 35.9 ms (280 bytes of
+// What bounds it (256 x 256, 4 CTAs of 512 threads): 64 slices x 500 iterations take 19.9 ms, 31.1
+// for pd_cluster.cuh's kernel in the same geometry.  On the way there: scalar transforms of one row after the other, state in tensor memory 35.9 ms (280 bytes of
 // spills, whose reloads miss the small L1); both rows packed 26.0; whole lines per gather instead of
-// 32-byte sectors (column-major units) 21.9; barriers split around independent work, D(k) in flight
-// during one, the field in thread order 20.0.  What is left is the exchange through distributed
-// shared memory (gather and scatter, a third of an iteration), the shared-memory wavefronts of the
-// column pass and the skew at four cluster barriers.
+// 32-byte sectors (column-major units) 21.8; barriers split around independent work, D(k) in flight
+// during one, the field in thread order 19.9.  What is left is the exchange through distributed
+// shared memory (gather, scatter and the barrier behind it, a quarter of an iteration), packed FP32
+// issue (a third), the shared-memory wavefronts of the column pass and the skew at the barriers.
 #pragma once
 
 #include <type_traits>
@@ -87,6 +86,7 @@ struct GeoPair {
     static_assert(!TMEM || (NT > 256 && (NT / 128) * TM_WORDS <= 512), "tensor-memory state: one CTA per SM");
     static_assert(E <= 32, "mask bits");
     static_assert(SMEM_BYTES <= 232448, "shared memory");
+    static_assert(!TMEM || 2 * (SMEM_BYTES + 1024) > 233472, "one tensor-memory CTA per SM");
     static constexpr int TMEM_COLS = 512;
 };
 
