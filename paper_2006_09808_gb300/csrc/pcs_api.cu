@@ -98,9 +98,12 @@ cudaError_t prepared(const pcs::KernelEntry* e, int* mc, int* aux) {
 
 namespace pcs {
 
-// The cheapest of the size's entries with a measured time: us per iteration, times the rounds when
-// the slices outnumber the resident clusters (the balanced schedule makes fractions of a round
-// count).  Without one: the first entry that answers to the kernel option.
+// us per iteration of S slices on mc resident clusters: the entry's time, times the rounds when the
+// slices outnumber the clusters (the balanced schedule makes fractions of a round count).
+static double entry_cost(const KernelEntry& e, int S, int mc) { return e.us * std::max(1.0, (double)S / mc); }
+
+// The cheapest (entry_cost) of the size's entries with a measured time.  Without one: the first entry
+// that answers to the kernel option.
 const KernelEntry* default_entry(int H, int W, int kernel, int S, int* max_clusters, int* max_clusters_aux,
                                  cudaError_t* err) {
     *err = cudaSuccess;
@@ -122,7 +125,7 @@ const KernelEntry* default_entry(int H, int W, int kernel, int S, int* max_clust
         if ((*err = prepared(&e, &mc, &aux)) != cudaSuccess) return first;
         mc = std::min(mc, sms / e.C);  // one CTA per SM
         if (mc < 1) continue;
-        const double cost = e.us * std::max(1.0, (double)S / mc);
+        const double cost = entry_cost(e, S, mc);
         if (!best || cost < best_cost) {
             best = &e;
             best_cost = cost;
@@ -916,6 +919,13 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
     t.W = c.W;
     double best = 1e300;
     pcs_status st = PCS_OK;
+    const pcs::KernelEntry* best_known = nullptr;  // the measured variant a context without options takes
+    {
+        int mc = 0, aux = 0;
+        cudaError_t ce = cudaSuccess;
+        const pcs::KernelEntry* k = pcs::default_entry(c.H, c.W, 0, S, &mc, &aux, &ce);
+        if (k && ce == cudaSuccess && k->us > 0.f) best_known = k;
+    }
     for (const auto& e : entries()) {
         if (e.H != c.H || e.W != c.W || t.n_candidates >= 8) continue;
         bool seen = false;  // the same kernel under the other kernel option
@@ -924,6 +934,13 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
             seen = seen || f.launch == e.launch;
         }
         if (seen) continue;
+        if (best_known && e.us > 0.f && &e != best_known) {
+            // measured variants that would take far longer than the best of them are not tried
+            int mc = 0, aux = 0, best_mc = 0;
+            if (prepared(&e, &mc, &aux) == cudaSuccess && prepared(best_known, &best_mc, &aux) == cudaSuccess &&
+                (mc < 1 || pcs::entry_cost(e, S, mc) > 1.5 * pcs::entry_cost(*best_known, S, std::max(1, best_mc))))
+                continue;
+        }
         pcs_options o = b->opt;
         o.cluster_size = e.C;
         o.kernel = e.resident ? 2 : 1;
