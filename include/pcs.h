@@ -198,6 +198,23 @@ PCS_API pcs_status pcs_schedule_plan(int S, int n_iter, int clusters, int *segme
                                      int *offsets);
 
 /*
+ * The cluster shape a call without variant options takes for a compiled size: of the shapes that
+ * give the same bits, the one whose measured time per iteration, times the rounds of its resident
+ * clusters, is least.  cluster_sizes[k], resident[k] (n of them): the clusters of each size the
+ * device holds at once (0 for a size not listed).  *cluster_size, *clusters receive the choice.
+ * Host only.  Errors: PCS_EINVAL, PCS_EUNSUPPORTED (no shape of the size is chosen this way).
+ */
+typedef struct pcs_shape_query {
+    int kernel;       /* as pcs_options.kernel */
+    int S;            /* slices of the call */
+    int whole_slices; /* 1: whole slices per cluster (pcs_solve_slices_noalloc, monitored solves); 0: the
+                         balanced schedule */
+    int sms;          /* SMs of the device */
+} pcs_shape_query;
+PCS_API pcs_status pcs_shape_plan(int H, int W, const pcs_shape_query *query, const int *cluster_sizes,
+                                  const int *resident, int n, int *cluster_size, int *clusters);
+
+/*
  * Test of the schedule's bounded wait: one warp waits on a flag that nothing
  * sets, with a limit of limit_cycles SM clock cycles, and *gave_up (host) is
  * set to 1 when the wait gave up.  Synchronises cuda_stream.

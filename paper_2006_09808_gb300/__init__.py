@@ -102,6 +102,10 @@ class pcs_tuning(ctypes.Structure):
         }
 
 
+class pcs_shape_query(ctypes.Structure):
+    _fields_ = [("kernel", ctypes.c_int), ("S", ctypes.c_int), ("whole_slices", ctypes.c_int), ("sms", ctypes.c_int)]
+
+
 class pcs_server_config(ctypes.Structure):
     _fields_ = [
         ("hbm_budget_bytes", ctypes.c_size_t),
@@ -165,6 +169,9 @@ def load_library(path: str = LIB_PATH):
         "pcs_check": (i, [vp]),
         "pcs_schedule_plan": (i, [i, i, i, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int),
                                   ctypes.POINTER(ctypes.c_int)]),
+        "pcs_shape_plan": (i, [i, i, ctypes.POINTER(pcs_shape_query), ctypes.POINTER(ctypes.c_int),
+                               ctypes.POINTER(ctypes.c_int), i, ctypes.POINTER(ctypes.c_int),
+                               ctypes.POINTER(ctypes.c_int)]),
         "pcs_selftest_wait": (i, [vp, ctypes.c_longlong, ctypes.POINTER(ctypes.c_int)]),
         "pcs_report": (i, [vp, vp, vp, i, d, vp, ctypes.POINTER(pcs_slice_report)]),
         "pcs_solve_slices_monitored": (i, [vp, vp, vp, i, d, d, d, i, i, d, vp, ctypes.POINTER(pcs_slice_report)]),
@@ -375,6 +382,17 @@ def pcs_schedule_plan(S: int, n_iter: int, clusters: int):
     off = (ctypes.c_int * (clusters + 1))()
     _check(lib.pcs_schedule_plan(S, n_iter, clusters, segs, ctypes.byref(n), off), "pcs_schedule_plan")
     return [tuple(segs[4 * k:4 * k + 4]) for k in range(n.value)], list(off)
+
+
+def pcs_shape_plan(H: int, W: int, S: int, resident: dict, sms: int = 152, **query):
+    """(cluster size, clusters) of a call without variant options; resident: {cluster size: resident clusters}."""
+    q = pcs_shape_query(S=S, sms=sms, **query)
+    n = len(resident)
+    arr = ctypes.c_int * max(1, n)
+    c, k = ctypes.c_int(), ctypes.c_int()
+    _check(load_library().pcs_shape_plan(H, W, ctypes.byref(q), arr(*resident.keys()), arr(*resident.values()), n,
+                                         ctypes.byref(c), ctypes.byref(k)), "pcs_shape_plan")
+    return c.value, k.value
 
 
 def pcs_check(ctx):

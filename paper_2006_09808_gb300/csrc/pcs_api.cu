@@ -98,42 +98,62 @@ cudaError_t prepared(const pcs::KernelEntry* e, int* mc, int* aux) {
 
 namespace pcs {
 
-// us per iteration of S slices on mc resident clusters: the entry's time, times the rounds when the
-// slices outnumber the clusters (the balanced schedule makes fractions of a round count).
-static double entry_cost(const KernelEntry& e, int S, int mc) { return e.us * std::max(1.0, (double)S / mc); }
+// us per iteration of the call on mc resident clusters of the entry: the entry's time, times the rounds
+// when the slices outnumber the clusters.  The balanced schedule makes fractions of a round count;
+// without it a cluster solves whole slices, and one slice more than the clusters costs a round (20
+// slices of 128 x 128 on 19 8-CTA clusters: 16.7 us per iteration, 9.3 on 4-CTA clusters).
+static double entry_cost(const KernelEntry& e, const ShapeCall& call, int mc) {
+    const double rounds = (double)call.S / mc;
+    return e.us * (call.whole ? std::ceil(rounds) : std::max(1.0, rounds));
+}
 
-// The cheapest (entry_cost) of the size's entries with a measured time.  Without one: the first entry
-// that answers to the kernel option.
-const KernelEntry* default_entry(int H, int W, int kernel, int S, int* max_clusters, int* max_clusters_aux,
-                                 cudaError_t* err) {
-    *err = cudaSuccess;
-    const KernelEntry* first = find_entry(H, W, 0, kernel);
-    if (!first) return nullptr;
-    if (first->us <= 0.f) {
-        *err = prepared(first, max_clusters, max_clusters_aux);
-        return first;
-    }
-    int dev = 0, sms = 0;
-    if ((*err = cudaGetDevice(&dev)) != cudaSuccess ||
-        (*err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return first;
+// The cheapest (entry_cost) of the size's entries with a measured time, given resident(entry), the
+// clusters the device holds of it.  NULL: none of them is resident.
+template <class F>
+static const KernelEntry* cheapest_entry(int H, int W, int is_resident, const ShapeCall& call, int sms, F resident,
+                                         int* max_clusters) {
     const KernelEntry* best = nullptr;
     double best_cost = 0.0;
     for (const auto& e : entries()) {
-        if (e.H != H || e.W != W || e.resident != first->resident || e.us <= 0.f) continue;
-        int mc = 0, aux = 0;
-        if ((*err = prepared(&e, &mc, &aux)) != cudaSuccess) return first;
-        mc = std::min(mc, sms / e.C);  // one CTA per SM
+        if (e.H != H || e.W != W || e.resident != is_resident || e.us <= 0.f) continue;
+        const int mc = std::min(resident(e), sms / e.C);  // one CTA per SM
         if (mc < 1) continue;
-        const double cost = entry_cost(e, S, mc);
+        const double cost = entry_cost(e, call, mc);
         if (!best || cost < best_cost) {
             best = &e;
             best_cost = cost;
             *max_clusters = mc;
-            *max_clusters_aux = aux;
         }
     }
-    if (best) return best;
+    return best;
+}
+
+// cheapest_entry on the current device.  For a size without a measured entry: the first entry that
+// answers to the kernel option.
+const KernelEntry* default_entry(int H, int W, int kernel, const ShapeCall& call, int* max_clusters,
+                                 int* max_clusters_aux, cudaError_t* err) {
+    *err = cudaSuccess;
+    const KernelEntry* first = find_entry(H, W, 0, kernel);
+    if (!first) return nullptr;
+    if (first->us > 0.f) {
+        int dev = 0, sms = 0;
+        if ((*err = cudaGetDevice(&dev)) != cudaSuccess ||
+            (*err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return first;
+        auto resident = [err](const KernelEntry& e) {
+            int mc = 0, aux = 0;
+            const cudaError_t pe = prepared(&e, &mc, &aux);
+            if (pe != cudaSuccess) *err = pe;
+            return mc;
+        };
+        const KernelEntry* best = cheapest_entry(H, W, first->resident, call, sms, resident, max_clusters);
+        if (*err != cudaSuccess) return first;
+        if (best) {
+            int mc = 0;
+            *err = prepared(best, &mc, max_clusters_aux);
+            return best;
+        }
+    }
     *err = prepared(first, max_clusters, max_clusters_aux);
     return first;
 }
@@ -345,7 +365,7 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
     if (!entry && ctx->by_count) {
         cudaError_t e = cudaSuccess;
         int aux = 0;
-        use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, S, &ncl, &aux, &e);
+        use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, {S, active != nullptr}, &ncl, &aux, &e);
         PCS_CUDA(e, "kernel attributes");
     }
     pcs::PDParams prm;
@@ -631,7 +651,7 @@ pcs_status pcs_create(pcs_ctx** out, int H, int W, int max_slices, const pcs_opt
     }
     c->by_count = o.cluster_size == 0 && o.threads == 0 && o.tile == 0 && entry->us > 0.f;
     if (c->by_count) {
-        c->entry = pcs::default_entry(H, W, o.kernel, max_slices, &c->max_clusters, &c->max_clusters_aux, &e);
+        c->entry = pcs::default_entry(H, W, o.kernel, {max_slices, false}, &c->max_clusters, &c->max_clusters_aux, &e);
     } else {
         e = prepared(entry, &c->max_clusters, &c->max_clusters_aux);
     }
@@ -681,6 +701,26 @@ pcs_status pcs_schedule_plan(int S, int n_iter, int clusters, int* segments, int
         segments[4 * k + 3] = segs[k].w;
     }
     for (int c = 0; c <= clusters; ++c) offsets[c] = off[c];
+    return PCS_OK;
+}
+
+pcs_status pcs_shape_plan(int H, int W, const pcs_shape_query* q, const int* cluster_sizes, const int* resident, int n,
+                          int* cluster_size, int* clusters) {
+    if (!q || !cluster_size || !clusters || n < 0 || (n > 0 && (!cluster_sizes || !resident)))
+        return fail(PCS_EINVAL, "NULL argument");
+    if (q->S < 1 || q->sms < 1 || q->kernel < 0 || q->kernel > 2) return fail(PCS_EINVAL, "S, sms or kernel");
+    const pcs::KernelEntry* first = find_entry(H, W, 0, q->kernel);
+    auto given = [&](const pcs::KernelEntry& e) {
+        for (int k = 0; k < n; ++k)
+            if (cluster_sizes[k] == e.C) return resident[k];
+        return 0;
+    };
+    const pcs::ShapeCall call{q->S, q->whole_slices != 0};
+    const pcs::KernelEntry* e = nullptr;
+    if (first && first->us > 0.f) e = pcs::cheapest_entry(H, W, first->resident, call, q->sms, given, clusters);
+    if (!e) return fail(PCS_EUNSUPPORTED, "no shape of %d x %d is chosen by the slice count", H, W);
+    *cluster_size = e->C;
+    *clusters = std::min(*clusters, q->S);
     return PCS_OK;
 }
 
@@ -817,7 +857,7 @@ pcs_status pcs_solve_slices_monitored(pcs_ctx* ctx, const float* field, const un
         if (ctx->by_count || ctx->entry->resident) {
             int aux = 0;
             cudaError_t ce = cudaSuccess;
-            e = pcs::default_entry(ctx->H, ctx->W, 1, S, &ncl, &aux, &ce);
+            e = pcs::default_entry(ctx->H, ctx->W, 1, {S, true}, &ncl, &aux, &ce);
             if (!e) return fail(PCS_EUNSUPPORTED, "no streaming kernel for %d x %d", ctx->H, ctx->W);
             PCS_CUDA(ce, "kernel attributes");
         }
@@ -923,7 +963,7 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
     {
         int mc = 0, aux = 0;
         cudaError_t ce = cudaSuccess;
-        const pcs::KernelEntry* k = pcs::default_entry(c.H, c.W, 0, S, &mc, &aux, &ce);
+        const pcs::KernelEntry* k = pcs::default_entry(c.H, c.W, 0, {S, false}, &mc, &aux, &ce);
         if (k && ce == cudaSuccess && k->us > 0.f) best_known = k;
     }
     for (const auto& e : entries()) {
@@ -938,7 +978,8 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
             // measured variants that would take far longer than the best of them are not tried
             int mc = 0, aux = 0, best_mc = 0;
             if (prepared(&e, &mc, &aux) == cudaSuccess && prepared(best_known, &best_mc, &aux) == cudaSuccess &&
-                (mc < 1 || pcs::entry_cost(e, S, mc) > 1.5 * pcs::entry_cost(*best_known, S, std::max(1, best_mc))))
+                (mc < 1 || pcs::entry_cost(e, {S, false}, mc) >
+                               1.5 * pcs::entry_cost(*best_known, {S, false}, std::max(1, best_mc))))
                 continue;
         }
         pcs_options o = b->opt;

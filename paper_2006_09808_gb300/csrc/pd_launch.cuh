@@ -198,10 +198,17 @@ const KernelEntry* entries_256(int* n);
 const KernelEntry* entries_384(int* n);
 const KernelEntry* entries_512(int* n);
 
-// The entry a call without variant options runs for S slices (kernel: 0 the size's default, 1, 2 the
-// option), how many of its clusters are resident (one CTA per SM) and how many of the auxiliary
-// kernels'; sets the kernels' attributes on the current device (cached).  NULL: none compiled.
-const KernelEntry* default_entry(int H, int W, int kernel, int S, int* max_clusters, int* max_clusters_aux,
-                                 cudaError_t* err);
+// What decides the shape of a call without variant options.
+struct ShapeCall {
+    int S;       // slices
+    bool whole;  // whole slices per cluster (no balanced schedule)
+};
+
+// The entry such a call runs (kernel: 0 the size's default, 1, 2 the option), how many of its clusters
+// are resident (one CTA per SM) and how many of the auxiliary kernels'.  The counts are kept per
+// device; the attributes are set when a count is first taken and by every pcs_create.  NULL: none
+// compiled.
+const KernelEntry* default_entry(int H, int W, int kernel, const ShapeCall& call, int* max_clusters,
+                                 int* max_clusters_aux, cudaError_t* err);
 
 }  // namespace pcs
