@@ -67,7 +67,10 @@ typedef enum pcs_status {
 typedef struct pcs_options {
     int b0_axis;       /* 0 = B0 along rows / y (default), 1 = along columns / x */
     int cluster_size;  /* 0 = library default for the slice size; else CTAs per slice (1,2,4,8,16) */
-    int max_clusters;  /* 0 = as many concurrent clusters as fit; else an upper bound (tuning) */
+    int max_clusters;  /* 0 = as many concurrent clusters as fit; else an upper bound.  Where the library
+                          chooses the cluster size it also bounds the SMs, to max_clusters times 1 (64x64),
+                          2 (192x192), 4 (128x128, 256x256, 384x384) or 8 (512x512), rounded up to a
+                          cluster of the size's smallest shape */
     int kernel;        /* 0 = library default; 1 = streaming (state in global memory);
                           2 = resident (state kept on chip for all iterations) */
     int threads;       /* 0 = library default; else threads per CTA of a compiled variant */
@@ -210,6 +213,7 @@ typedef struct pcs_shape_query {
     int whole_slices; /* 1: whole slices per cluster (pcs_solve_slices_noalloc, monitored solves); 0: the
                          balanced schedule */
     int sms;          /* SMs of the device */
+    int max_clusters; /* as pcs_options.max_clusters */
 } pcs_shape_query;
 PCS_API pcs_status pcs_shape_plan(int H, int W, const pcs_shape_query *query, const int *cluster_sizes,
                                   const int *resident, int n, int *cluster_size, int *clusters);

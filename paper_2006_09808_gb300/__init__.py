@@ -103,7 +103,8 @@ class pcs_tuning(ctypes.Structure):
 
 
 class pcs_shape_query(ctypes.Structure):
-    _fields_ = [("kernel", ctypes.c_int), ("S", ctypes.c_int), ("whole_slices", ctypes.c_int), ("sms", ctypes.c_int)]
+    _fields_ = [("kernel", ctypes.c_int), ("S", ctypes.c_int), ("whole_slices", ctypes.c_int), ("sms", ctypes.c_int),
+                ("max_clusters", ctypes.c_int)]
 
 
 class pcs_server_config(ctypes.Structure):

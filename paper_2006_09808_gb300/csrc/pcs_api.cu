@@ -107,16 +107,32 @@ static double entry_cost(const KernelEntry& e, const ShapeCall& call, int mc) {
     return e.us * (call.whole ? std::ceil(rounds) : std::max(1.0, rounds));
 }
 
+// Clusters of the entry that a call may use of `resident` ones: one CTA per SM, and with max_clusters
+// at most that many clusters on at most as many SMs as that many of the size's base clusters (aux_C
+// CTAs each).  A caller that leaves SMs to other work by it keeps them: one slice of 256 x 256 with
+// max_clusters = 1 runs on 4 SMs and not in a 16-CTA cluster.  The size's smallest shape rounds up to
+// whole clusters (192, 384 and 512: 3, 8 and 16 CTAs on a base of 2, 4 and 8).
+static int usable_clusters(const KernelEntry& e, bool smallest, int resident, int sms, int cap) {
+    const int mc = std::min(resident, sms / e.C);
+    if (cap <= 0) return mc;
+    const long long sm = (long long)cap * e.aux_C;
+    return (int)std::min<long long>({mc, cap, (sm + (smallest ? e.C - 1 : 0)) / e.C});
+}
+
 // The cheapest (entry_cost) of the size's entries with a measured time, given resident(entry), the
 // clusters the device holds of it.  NULL: none of them is resident.
 template <class F>
 static const KernelEntry* cheapest_entry(int H, int W, int is_resident, const ShapeCall& call, int sms, F resident,
                                          int* max_clusters) {
+    auto candidate = [&](const KernelEntry& e) { return e.H == H && e.W == W && e.resident == is_resident && e.us > 0.f; };
+    int least_C = 0;
+    for (const auto& e : entries())
+        if (candidate(e) && (least_C == 0 || e.C < least_C) && resident(e) >= 1) least_C = e.C;
     const KernelEntry* best = nullptr;
     double best_cost = 0.0;
     for (const auto& e : entries()) {
-        if (e.H != H || e.W != W || e.resident != is_resident || e.us <= 0.f) continue;
-        const int mc = std::min(resident(e), sms / e.C);  // one CTA per SM
+        if (!candidate(e)) continue;
+        const int mc = usable_clusters(e, e.C == least_C, resident(e), sms, call.cap);
         if (mc < 1) continue;
         const double cost = entry_cost(e, call, mc);
         if (!best || cost < best_cost) {
@@ -365,7 +381,7 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
     if (!entry && ctx->by_count) {
         cudaError_t e = cudaSuccess;
         int aux = 0;
-        use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, {S, active != nullptr}, &ncl, &aux, &e);
+        use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, {S, active != nullptr, ctx->opt.max_clusters}, &ncl, &aux, &e);
         PCS_CUDA(e, "kernel attributes");
     }
     pcs::PDParams prm;
@@ -651,7 +667,7 @@ pcs_status pcs_create(pcs_ctx** out, int H, int W, int max_slices, const pcs_opt
     }
     c->by_count = o.cluster_size == 0 && o.threads == 0 && o.tile == 0 && entry->us > 0.f;
     if (c->by_count) {
-        c->entry = pcs::default_entry(H, W, o.kernel, {max_slices, false}, &c->max_clusters, &c->max_clusters_aux, &e);
+        c->entry = pcs::default_entry(H, W, o.kernel, {max_slices, false, o.max_clusters}, &c->max_clusters, &c->max_clusters_aux, &e);
     } else {
         e = prepared(entry, &c->max_clusters, &c->max_clusters_aux);
     }
@@ -715,7 +731,7 @@ pcs_status pcs_shape_plan(int H, int W, const pcs_shape_query* q, const int* clu
             if (cluster_sizes[k] == e.C) return resident[k];
         return 0;
     };
-    const pcs::ShapeCall call{q->S, q->whole_slices != 0};
+    const pcs::ShapeCall call{q->S, q->whole_slices != 0, q->max_clusters};
     const pcs::KernelEntry* e = nullptr;
     if (first && first->us > 0.f) e = pcs::cheapest_entry(H, W, first->resident, call, q->sms, given, clusters);
     if (!e) return fail(PCS_EUNSUPPORTED, "no shape of %d x %d is chosen by the slice count", H, W);
@@ -857,7 +873,7 @@ pcs_status pcs_solve_slices_monitored(pcs_ctx* ctx, const float* field, const un
         if (ctx->by_count || ctx->entry->resident) {
             int aux = 0;
             cudaError_t ce = cudaSuccess;
-            e = pcs::default_entry(ctx->H, ctx->W, 1, {S, true}, &ncl, &aux, &ce);
+            e = pcs::default_entry(ctx->H, ctx->W, 1, {S, true, ctx->opt.max_clusters}, &ncl, &aux, &ce);
             if (!e) return fail(PCS_EUNSUPPORTED, "no streaming kernel for %d x %d", ctx->H, ctx->W);
             PCS_CUDA(ce, "kernel attributes");
         }
@@ -959,11 +975,12 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
     t.W = c.W;
     double best = 1e300;
     pcs_status st = PCS_OK;
+    const pcs::ShapeCall call{S, false, b->opt.max_clusters};
     const pcs::KernelEntry* best_known = nullptr;  // the measured variant a context without options takes
     {
         int mc = 0, aux = 0;
         cudaError_t ce = cudaSuccess;
-        const pcs::KernelEntry* k = pcs::default_entry(c.H, c.W, 0, {S, false}, &mc, &aux, &ce);
+        const pcs::KernelEntry* k = pcs::default_entry(c.H, c.W, 0, call, &mc, &aux, &ce);
         if (k && ce == cudaSuccess && k->us > 0.f) best_known = k;
     }
     for (const auto& e : entries()) {
@@ -977,10 +994,14 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
         if (best_known && e.us > 0.f && &e != best_known) {
             // measured variants that would take far longer than the best of them are not tried
             int mc = 0, aux = 0, best_mc = 0;
-            if (prepared(&e, &mc, &aux) == cudaSuccess && prepared(best_known, &best_mc, &aux) == cudaSuccess &&
-                (mc < 1 || pcs::entry_cost(e, {S, false}, mc) >
-                               1.5 * pcs::entry_cost(*best_known, {S, false}, std::max(1, best_mc))))
-                continue;
+            if (prepared(&e, &mc, &aux) == cudaSuccess && prepared(best_known, &best_mc, &aux) == cudaSuccess) {
+                if (call.cap > 0) {  // the option's own meaning: clusters
+                    mc = std::min(mc, call.cap);
+                    best_mc = std::min(best_mc, call.cap);
+                }
+                if (mc < 1 || pcs::entry_cost(e, call, mc) > 1.5 * pcs::entry_cost(*best_known, call, std::max(1, best_mc)))
+                    continue;
+            }
         }
         pcs_options o = b->opt;
         o.cluster_size = e.C;

@@ -202,6 +202,7 @@ const KernelEntry* entries_512(int* n);
 struct ShapeCall {
     int S;       // slices
     bool whole;  // whole slices per cluster (no balanced schedule)
+    int cap;     // pcs_options.max_clusters
 };
 
 // The entry such a call runs (kernel: 0 the size's default, 1, 2 the option), how many of its clusters

@@ -38,6 +38,26 @@ def test_whole_slices_cost_whole_rounds(H, S, balanced, whole):
     assert plan(H, S, whole_slices=1) == (whole, min(S, RESIDENT[H][whole]))
 
 
+@pytest.mark.parametrize("H,base", [(64, 1), (128, 4), (192, 2), (256, 4), (384, 4), (512, 8)])
+def test_max_clusters_bounds_the_sms(H, base):
+    """At most max_clusters clusters on at most that many times the base's SMs; only the smallest shape rounds up."""
+    least = min(c for c in RESIDENT[H] if H != 128 or c > 1)  # 128's one-CTA shape is by option only
+    for cap in (1, 2, 3, 5, 8, 16, 36, 200):
+        for S in (1, 2, 7, 20, 64):
+            for whole in (0, 1):
+                c, k = plan(H, S, max_clusters=cap, whole_slices=whole)
+                assert 1 <= k <= min(cap, S, RESIDENT[H][c])
+                assert c * k <= cap * base or (c == least and c * (k - 1) < cap * base)
+    assert plan(H, 64, max_clusters=1000) == plan(H, 64)
+
+
+def test_max_clusters_choices():
+    assert plan(256, 1, max_clusters=1) == (4, 1)
+    assert plan(256, 1, max_clusters=4) == (16, 1)
+    assert plan(256, 64, max_clusters=8) == (4, 8)
+    assert plan(128, 64, max_clusters=8) == (4, 8)  # not 8 of the 2-CTA shape
+
+
 def test_arguments():
     for H in RESIDENT:
         c, k = plan(H, 1)
