@@ -4,11 +4,12 @@
 namespace pcs {
 using Aux = Geo<192, 192, 2, 2>;
 static const KernelEntry k_entries[] = {
-    // 3-CTA clusters: 22.4 us per iteration of up to 48 slices, 47 for the half-spectrum kernel below;
-    // larger clusters for fewer slices: 15.1 us (up to 20) and 12.0 us (up to 8)
-    make_pair_entry<GeoPair<192, 3, 512, true>, Aux>(22.4f),
-    make_pair_entry<GeoPair<192, 6, 256, false>, Aux>(15.1f),
-    make_pair_entry<GeoPair<192, 12, 128, false>, Aux>(12.0f),
+    // us per iteration (isotropic weighted): 12-CTA clusters 12.4 (16.5) for up to 8 slices, 3-CTA 22.8
+    // (27.6) for up to 40, 6-CTA 15.4 (19.3) for up to 21 and, on the balanced schedule, 16.5 (21.1) for
+    // 24; 47 (57) for the half-spectrum kernel below
+    make_pair_entry<GeoPair<192, 3, 512, true>, Aux>(22.8f),
+    make_pair_entry<GeoPair<192, 6, 256, false>, Aux>(15.4f),
+    make_pair_entry<GeoPair<192, 12, 128, false>, Aux>(12.4f),
     make_entry<Geo<192, 192, 2, 2>>(),
 };
 const KernelEntry* entries_192(int* n) {

@@ -4,11 +4,12 @@
 namespace pcs {
 using Aux = Geo<256, 256, 4, 1, 512>;
 static const KernelEntry k_entries[] = {
-    // 23.1 us per iteration of up to 36 slices (35 for the half-spectrum kernel in the same geometry,
-    // Geo<256, 256, 4, 1, 512>); larger clusters for fewer slices: 17.7 us for up to 15, 13.6 us for up to 8
-    make_pair_entry<GeoPair<256, 4, 512, true>, Aux>(23.1f),
-    make_pair_entry<GeoPair<256, 8, 256, false>, Aux>(17.7f),
-    make_pair_entry<GeoPair<256, 16, 128, false>, Aux>(13.6f),
+    // us per iteration (isotropic weighted): 4-CTA clusters 22.7 (29.6) for up to 36 slices (35 for the
+    // half-spectrum kernel in the same geometry, Geo<256, 256, 4, 1, 512>); larger clusters for fewer
+    // slices: 8-CTA 16.5 (23.2) for up to 15, 16-CTA 14.2 (20.9) for up to 7 or 8 (by device)
+    make_pair_entry<GeoPair<256, 4, 512, true>, Aux>(22.7f),
+    make_pair_entry<GeoPair<256, 8, 256, false>, Aux>(16.5f),
+    make_pair_entry<GeoPair<256, 16, 128, false>, Aux>(14.2f),
     make_entry<Geo<256, 256, 4, 2>>(),
     make_resident_entry<GeoRes<256, 256, 8>>(),
     make_entry<Geo<256, 256, 2, 1>>(),

@@ -27,9 +27,11 @@ struct KernelEntry {
     // the balanced-schedule instantiation of the iteration kernel (NULL for pd_resident_kernel)
     cudaError_t (*launch_sched)(const PDParams& prm, int n_clusters, cudaStream_t stream);
     int aux_C;     // cluster size of the diagnostics and power iteration
-    // Measured us per iteration with at most one CTA per SM; the entries of a size that have it give
-    // bit-identical results, and contexts without variant options take the cheapest for the call's
-    // slice count (default_entry in pcs_api.cu).  0: only by option or autotuner.
+    // Measured us per iteration with at most one CTA per SM, all clusters at work (anisotropic and
+    // unweighted; by isotropic weighted times the choice would be the same or within 8%).  The entries
+    // of a size that have it give bit-identical results, and contexts without variant options take the
+    // cheapest for the call's slice count (default_entry in pcs_api.cu).  0: only by option or
+    // autotuner.
     float us;
 };
 

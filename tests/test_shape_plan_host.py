@@ -29,12 +29,11 @@ def plan(H, S, **query):
 @pytest.mark.parametrize("H,S,balanced,whole", [
     # one slice more than the larger clusters hold: a fraction of a round on the balanced schedule,
     # a whole round without it
-    (128, 19, 8, 8), (128, 21, None, 4), (192, 8, 12, 12), (192, 9, 12, 6), (256, 8, 16, 16), (256, 9, 16, 8),
+    (128, 19, 8, 8), (128, 20, 4, 4), (192, 8, 12, 12), (192, 9, 12, 6), (256, 8, 16, 16), (256, 9, 16, 8),
     (256, 15, 8, 8), (256, 16, 8, 4), (256, 37, 4, 4),
 ])
 def test_whole_slices_cost_whole_rounds(H, S, balanced, whole):
-    if balanced:
-        assert plan(H, S) == (balanced, min(S, RESIDENT[H][balanced]))
+    assert plan(H, S) == (balanced, min(S, RESIDENT[H][balanced]))
     assert plan(H, S, whole_slices=1) == (whole, min(S, RESIDENT[H][whole]))
 
 
