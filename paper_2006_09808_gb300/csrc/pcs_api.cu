@@ -120,7 +120,8 @@ static int usable_clusters(const KernelEntry& e, bool smallest, int resident, in
 }
 
 // The cheapest (entry_cost) of the size's entries with a measured time, given resident(entry), the
-// clusters the device holds of it.  NULL: none of them is resident.
+// clusters the device holds of it.  Where it holds none of them (a part of a GPU without room for a 16-CTA
+// cluster), the first other entry of the kind that it does hold.  NULL: none.
 template <class F>
 static const KernelEntry* cheapest_entry(int H, int W, int is_resident, const ShapeCall& call, int sms, F resident,
                                          int* max_clusters) {
@@ -141,7 +142,13 @@ static const KernelEntry* cheapest_entry(int H, int W, int is_resident, const Sh
             *max_clusters = mc;
         }
     }
-    return best;
+    if (best) return best;
+    for (const auto& e : entries())
+        if (e.H == H && e.W == W && e.resident == is_resident && e.us <= 0.f && resident(e) >= 1) {
+            *max_clusters = call.cap > 0 ? std::min(resident(e), call.cap) : resident(e);
+            return &e;
+        }
+    return nullptr;
 }
 
 // cheapest_entry on the current device.  For a size without a measured entry: the first entry that

@@ -57,6 +57,15 @@ def test_max_clusters_choices():
     assert plan(128, 64, max_clusters=8) == (4, 8)  # not 8 of the 2-CTA shape
 
 
+def test_device_without_room_for_the_chosen_shapes():
+    """A part of a GPU that holds no 16-CTA (or 8-CTA) cluster solves with a half-spectrum variant."""
+    assert pcs.pcs_shape_plan(512, 512, 5, {16: 0, 8: 2}) == (8, 2)
+    assert pcs.pcs_shape_plan(512, 512, 5, {16: 1, 8: 2}, sms=15) == (8, 2)
+    assert pcs.pcs_shape_plan(384, 384, 5, {8: 0, 4: 3}, max_clusters=2) == (4, 2)
+    with pytest.raises(pcs.PcsError):
+        pcs.pcs_shape_plan(512, 512, 5, {16: 0, 8: 0})
+
+
 def test_arguments():
     for H in RESIDENT:
         c, k = plan(H, 1)
