@@ -145,7 +145,8 @@ PCS_API pcs_status pcs_set_stream(pcs_ctx *ctx, void *cuda_stream);
  * All device pointers must be 16-byte aligned.  Slices are independent: the
  * result for a slice does not depend on the other slices in the call.  A
  * context whose options leave cluster_size, threads and tile at 0 takes, for
- * each call, the cluster size that suits S; those of a size give the same bits.
+ * each call, the cluster size that suits S and what else is in flight
+ * (pcs_last_variant); those of a size give the same bits.
  * Errors: PCS_EINVAL, PCS_ECUDA.
  */
 PCS_API pcs_status pcs_solve_slices(pcs_ctx *ctx, const float *field, const unsigned char *mask, int S,
@@ -214,9 +215,21 @@ typedef struct pcs_shape_query {
                          balanced schedule */
     int sms;          /* SMs of the device */
     int max_clusters; /* as pcs_options.max_clusters */
+    int solves;       /* other solves in flight (see pcs_last_variant) ... */
+    int pad;
+    double in_flight; /* ... and their slices, in units of this size's pixels */
 } pcs_shape_query;
 PCS_API pcs_status pcs_shape_plan(int H, int W, const pcs_shape_query *query, const int *cluster_sizes,
                                   const int *resident, int n, int *cluster_size, int *clusters);
+
+/*
+ * The kernel variant and the clusters of the context's last solve (zeros before the first, and for
+ * any-size contexts).  A context without variant options chooses them for each call from its slice
+ * count and from the slices of solves that other contexts of the process have in flight on other
+ * streams of the device: alone, few slices run in large clusters (least time); beside other solves in
+ * small ones (least SM time).  A context with use_graph keeps the shape its graph was captured with.
+ */
+PCS_API pcs_status pcs_last_variant(pcs_ctx *ctx, int *cluster_size, int *threads, int *tile, int *clusters);
 
 /*
  * Test of the schedule's bounded wait: one warp waits on a flag that nothing

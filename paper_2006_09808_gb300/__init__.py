@@ -104,7 +104,8 @@ class pcs_tuning(ctypes.Structure):
 
 class pcs_shape_query(ctypes.Structure):
     _fields_ = [("kernel", ctypes.c_int), ("S", ctypes.c_int), ("whole_slices", ctypes.c_int), ("sms", ctypes.c_int),
-                ("max_clusters", ctypes.c_int)]
+                ("max_clusters", ctypes.c_int), ("solves", ctypes.c_int), ("pad", ctypes.c_int),
+                ("in_flight", ctypes.c_double)]
 
 
 class pcs_server_config(ctypes.Structure):
@@ -173,6 +174,7 @@ def load_library(path: str = LIB_PATH):
         "pcs_shape_plan": (i, [i, i, ctypes.POINTER(pcs_shape_query), ctypes.POINTER(ctypes.c_int),
                                ctypes.POINTER(ctypes.c_int), i, ctypes.POINTER(ctypes.c_int),
                                ctypes.POINTER(ctypes.c_int)]),
+        "pcs_last_variant": (i, [vp] + [ctypes.POINTER(ctypes.c_int)] * 4),
         "pcs_selftest_wait": (i, [vp, ctypes.c_longlong, ctypes.POINTER(ctypes.c_int)]),
         "pcs_report": (i, [vp, vp, vp, i, d, vp, ctypes.POINTER(pcs_slice_report)]),
         "pcs_solve_slices_monitored": (i, [vp, vp, vp, i, d, d, d, i, i, d, vp, ctypes.POINTER(pcs_slice_report)]),
@@ -394,6 +396,12 @@ def pcs_shape_plan(H: int, W: int, S: int, resident: dict, sms: int = 152, **que
     _check(load_library().pcs_shape_plan(H, W, ctypes.byref(q), arr(*resident.keys()), arr(*resident.values()), n,
                                          ctypes.byref(c), ctypes.byref(k)), "pcs_shape_plan")
     return c.value, k.value
+
+
+def pcs_last_variant(ctx):
+    v = [ctypes.c_int() for _ in range(4)]
+    _check(load_library().pcs_last_variant(ctx, *(ctypes.byref(x) for x in v)), "pcs_last_variant")
+    return dict(zip(("cluster_size", "threads", "tile", "clusters"), (x.value for x in v)))
 
 
 def pcs_check(ctx):

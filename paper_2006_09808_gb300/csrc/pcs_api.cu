@@ -101,10 +101,17 @@ namespace pcs {
 // us per iteration of the call on mc resident clusters of the entry: the entry's time, times the rounds
 // when the slices outnumber the clusters.  The balanced schedule makes fractions of a round count;
 // without it a cluster solves whole slices, and one slice more than the clusters costs a round (20
-// slices of 128 x 128 on 19 8-CTA clusters: 16.7 us per iteration, 9.3 on 4-CTA clusters).
+// slices of 128 x 128 on 19 8-CTA clusters: 16.7 us per iteration, 9.3 on 4-CTA clusters).  Slices of
+// other solves in flight share the clusters in fractions of a round: a slice alone is quickest in a
+// large cluster, but many calls at once in small ones, which cost fewer SM-us per slice (24 one-slice
+// contexts of 256 x 256 on 24 streams: 49 us per iteration in 16-CTA clusters, 22.6 in 4-CTA ones).  The
+// device runs the streams of up to 32 of them at once; more wait for one another (36 streams take the
+// time of two solves in 3-CTA clusters at 192 x 192, 45 us, but 32 in larger ones).
 static double entry_cost(const KernelEntry& e, const ShapeCall& call, int mc) {
+    constexpr int kStreams = 32;
     const double rounds = (double)call.S / mc;
-    return e.us * (call.whole ? std::ceil(rounds) : std::max(1.0, rounds));
+    const double own = call.whole ? std::ceil(rounds) : std::max(1.0, rounds);
+    return e.us * std::max(own * (1 + call.solves / kStreams), (call.S + call.in_flight) / mc);
 }
 
 // Clusters of the entry that a call may use of `resident` ones: one CTA per SM, and with max_clusters
@@ -299,13 +306,78 @@ struct pcs_ctx {
     pcs::PDParams graph_prm{};
     int graph_ncl = 0;
     const pcs::KernelEntry* graph_entry = nullptr;
+    pcs::PDParams graph_args{};  // graph_prm without the schedule
+    // the last solve: its variant and clusters (pcs_last_variant)
+    const pcs::KernelEntry* ran_entry = nullptr;
+    int ran_clusters = 0;
+    // the last solve enqueued, for the other contexts' choice of shape (guarded by live_mu): an event behind
+    // it, its stream and slices (0: none, or known to be done); contexts of one group (the size classes
+    // of a batch, solved in turn) do not count each other
+    cudaEvent_t ran = nullptr;
+    cudaStream_t ran_stream = nullptr;
+    int ran_S = 0;
+    const void* group = nullptr;
     std::mutex mu;
 };
 
 namespace {
 
+// Contexts of the process, for count_in_flight.
+std::mutex live_mu;
+std::vector<pcs_ctx*>& live() {
+    static auto* v = new std::vector<pcs_ctx*>;  // outlives every static object that destroys a context
+    return *v;
+}
+
+// Whether the context's stream is being captured (its work does not run now), or cannot be asked.
+bool capturing(const pcs_ctx* c) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return true;
+}
+
+// The last solves that other contexts enqueued on other streams of the device and that have not
+// finished: how many, and their slices in units of this context's slice pixels.
+void count_in_flight(const pcs_ctx* c, pcs::ShapeCall* call) {
+    std::lock_guard<std::mutex> lk(live_mu);
+    // an event query is allowed beside another thread's stream capture only in this thread mode
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return;
+    for (pcs_ctx* o : live()) {
+        if (o == c || o->ran_S == 0 || o->device != c->device || o->ran_stream == c->stream ||
+            (o->group && o->group == c->group))
+            continue;
+        const cudaError_t e = cudaEventQuery(o->ran);
+        if (e == cudaErrorNotReady) {
+            ++call->solves;
+            call->in_flight += (double)o->ran_S * o->H * o->W / ((double)c->H * c->W);
+        } else {
+            o->ran_S = 0;
+        }
+        if (e != cudaSuccess) (void)cudaGetLastError();  // "not ready" is no error of the caller's
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+// After a solve of S slices was enqueued.
+void note_solve(pcs_ctx* c, int S, const pcs::KernelEntry* entry, int clusters) {
+    c->ran_entry = entry;
+    c->ran_clusters = clusters;
+    if (!c->ran || capturing(c)) return;
+    std::lock_guard<std::mutex> lk(live_mu);
+    c->ran_stream = c->stream;
+    c->ran_S = cudaEventRecord(c->ran, c->stream) == cudaSuccess ? S : 0;
+    if (c->ran_S == 0) (void)cudaGetLastError();
+}
+
 void free_ctx(pcs_ctx* c) {
     if (!c) return;
+    {
+        std::lock_guard<std::mutex> lk(live_mu);
+        live().erase(std::remove(live().begin(), live().end(), c), live().end());
+    }
+    if (c->ran) cudaEventDestroy(c->ran);
     void* ptrs[] = {c->dtab,     c->ddtab,  c->twid,     c->chibar, c->p,  c->qx,   c->qy,
                     c->st_field, c->st_mask, c->st_chi,  c->partials, c->Ldev, c->xa,  c->xb,
                     c->active,   c->sched,   c->sched_off, c->seg_flags, c->err};
@@ -379,18 +451,11 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
                                   lambda, tau, sigma, n_iter, ctx->stream, resume, active, inv_den_slice,
                                   nullptr),
                  "launch of the any-size kernels");
+        note_solve(ctx, S, nullptr, 0);
         ctx->last_iters = n_iter;
         return PCS_OK;
     }
     PCS_CUDA(cudaSetDevice(ctx->device), "cudaSetDevice");
-    const pcs::KernelEntry* use = entry ? entry : ctx->entry;
-    int ncl = ncl_override > 0 ? ncl_override : ctx->max_clusters;
-    if (!entry && ctx->by_count) {
-        cudaError_t e = cudaSuccess;
-        int aux = 0;
-        use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, {S, active != nullptr, ctx->opt.max_clusters}, &ncl, &aux, &e);
-        PCS_CUDA(e, "kernel attributes");
-    }
     pcs::PDParams prm;
     std::memset(&prm, 0, sizeof(prm));  // padding too: the graph cache compares whole structs
     prm.field = field;
@@ -413,6 +478,22 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
     prm.resume = resume;
     prm.tv_iso = ctx->opt.tv;
     prm.weight = weight;
+    const pcs::PDParams args = prm;  // what the caller asked for
+    const pcs::KernelEntry* use = entry ? entry : ctx->entry;
+    int ncl = ncl_override > 0 ? ncl_override : ctx->max_clusters;
+    if (!entry && ctx->by_count) {
+        if (ctx->opt.use_graph && ctx->graph_exec && std::memcmp(&args, &ctx->graph_args, sizeof(args)) == 0) {
+            use = ctx->graph_entry;  // a captured solve keeps its shape
+            ncl = ctx->graph_ncl;
+        } else {
+            cudaError_t e = cudaSuccess;
+            int aux = 0;
+            pcs::ShapeCall call{S, active != nullptr, ctx->opt.max_clusters, 0, 0.0};
+            if (!capturing(ctx)) count_in_flight(ctx, &call);
+            use = pcs::default_entry(ctx->H, ctx->W, ctx->opt.kernel, call, &ncl, &aux, &e);
+            PCS_CUDA(e, "kernel attributes");
+        }
+    }
     if (ctx->opt.max_clusters > 0 && ctx->opt.max_clusters < ncl) ncl = ctx->opt.max_clusters;
     if (ncl > S) ncl = S;
     if (ncl < 1) ncl = 1;
@@ -455,6 +536,7 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
     };
     if (entry && entry != ctx->entry) {  // another variant of the same size (monitored solves)
         PCS_CUDA(launch(use), "launch of the primal-dual kernel");
+        note_solve(ctx, S, use, ncl);
         ctx->last_iters = n_iter;
         return PCS_OK;
     }
@@ -479,6 +561,7 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
             ctx->graph = g;
             PCS_CUDA(cudaGraphInstantiate(&ctx->graph_exec, g, 0), "graph instantiate");
             ctx->graph_prm = prm;
+            ctx->graph_args = args;
             ctx->graph_ncl = ncl;
             ctx->graph_entry = use;
         }
@@ -486,6 +569,7 @@ pcs_status launch_solve(pcs_ctx* ctx, const float* field, const unsigned char* m
     } else {
         PCS_CUDA(launch(use), "launch of the primal-dual kernel");
     }
+    note_solve(ctx, S, use, ncl);
     ctx->last_iters = n_iter;
     return PCS_OK;
 }
@@ -659,6 +743,12 @@ pcs_status pcs_create(pcs_ctx** out, int H, int W, int max_slices, const pcs_opt
         return st;
     };
     if ((e = cudaGetDevice(&c->device)) != cudaSuccess) return bail(cuda_fail(e, "cudaGetDevice"));
+    if ((e = cudaEventCreateWithFlags(&c->ran, cudaEventDisableTiming)) != cudaSuccess)
+        return bail(cuda_fail(e, "event"));
+    {
+        std::lock_guard<std::mutex> lk(live_mu);
+        live().push_back(c);
+    }
     if (any_size) {
         // the any-size row/column kernels: their own tables and spectrum; the state as below
         const size_t n = slice_elems(c) * (size_t)max_slices;
@@ -674,7 +764,8 @@ pcs_status pcs_create(pcs_ctx** out, int H, int W, int max_slices, const pcs_opt
     }
     c->by_count = o.cluster_size == 0 && o.threads == 0 && o.tile == 0 && entry->us > 0.f;
     if (c->by_count) {
-        c->entry = pcs::default_entry(H, W, o.kernel, {max_slices, false, o.max_clusters}, &c->max_clusters, &c->max_clusters_aux, &e);
+        c->entry = pcs::default_entry(H, W, o.kernel, {max_slices, false, o.max_clusters, 0, 0.0}, &c->max_clusters,
+                                      &c->max_clusters_aux, &e);
     } else {
         e = prepared(entry, &c->max_clusters, &c->max_clusters_aux);
     }
@@ -731,19 +822,30 @@ pcs_status pcs_shape_plan(int H, int W, const pcs_shape_query* q, const int* clu
                           int* cluster_size, int* clusters) {
     if (!q || !cluster_size || !clusters || n < 0 || (n > 0 && (!cluster_sizes || !resident)))
         return fail(PCS_EINVAL, "NULL argument");
-    if (q->S < 1 || q->sms < 1 || q->kernel < 0 || q->kernel > 2) return fail(PCS_EINVAL, "S, sms or kernel");
+    if (q->S < 1 || q->sms < 1 || q->kernel < 0 || q->kernel > 2 || q->solves < 0 || !(q->in_flight >= 0.0))
+        return fail(PCS_EINVAL, "S, sms, kernel, solves or in_flight");
     const pcs::KernelEntry* first = find_entry(H, W, 0, q->kernel);
     auto given = [&](const pcs::KernelEntry& e) {
         for (int k = 0; k < n; ++k)
             if (cluster_sizes[k] == e.C) return resident[k];
         return 0;
     };
-    const pcs::ShapeCall call{q->S, q->whole_slices != 0, q->max_clusters};
+    const pcs::ShapeCall call{q->S, q->whole_slices != 0, q->max_clusters, q->solves, q->in_flight};
     const pcs::KernelEntry* e = nullptr;
     if (first && first->us > 0.f) e = pcs::cheapest_entry(H, W, first->resident, call, q->sms, given, clusters);
     if (!e) return fail(PCS_EUNSUPPORTED, "no shape of %d x %d is chosen by the slice count", H, W);
     *cluster_size = e->C;
     *clusters = std::min(*clusters, q->S);
+    return PCS_OK;
+}
+
+pcs_status pcs_last_variant(pcs_ctx* ctx, int* cluster_size, int* threads, int* tile, int* clusters) {
+    if (!ctx || !cluster_size || !threads || !tile || !clusters) return fail(PCS_EINVAL, "NULL argument");
+    const pcs::KernelEntry* e = ctx->ran_entry;
+    *cluster_size = e ? e->C : 0;
+    *threads = e ? e->threads : 0;
+    *tile = e ? e->tile : 0;
+    *clusters = e ? ctx->ran_clusters : 0;
     return PCS_OK;
 }
 
@@ -880,7 +982,9 @@ pcs_status pcs_solve_slices_monitored(pcs_ctx* ctx, const float* field, const un
         if (ctx->by_count || ctx->entry->resident) {
             int aux = 0;
             cudaError_t ce = cudaSuccess;
-            e = pcs::default_entry(ctx->H, ctx->W, 1, {S, true, ctx->opt.max_clusters}, &ncl, &aux, &ce);
+            pcs::ShapeCall call{S, true, ctx->opt.max_clusters, 0, 0.0};
+            count_in_flight(ctx, &call);
+            e = pcs::default_entry(ctx->H, ctx->W, 1, call, &ncl, &aux, &ce);
             if (!e) return fail(PCS_EUNSUPPORTED, "no streaming kernel for %d x %d", ctx->H, ctx->W);
             PCS_CUDA(ce, "kernel attributes");
         }
@@ -982,7 +1086,7 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
     t.W = c.W;
     double best = 1e300;
     pcs_status st = PCS_OK;
-    const pcs::ShapeCall call{S, false, b->opt.max_clusters};
+    const pcs::ShapeCall call{S, false, b->opt.max_clusters, 0, 0.0};
     const pcs::KernelEntry* best_known = nullptr;  // the measured variant a context without options takes
     {
         int mc = 0, aux = 0;
@@ -1087,6 +1191,7 @@ pcs_status prepare_class(pcs_batch* b, pcs_batch::Class& c, int S) {
     }
     pcs_status st = pcs_create(&c.ctx, c.H, c.W, cap, &o, c.stream);
     if (st != PCS_OK) return st;
+    c.ctx->group = b;
     const size_t n = (size_t)cap * c.H * c.W;
     PCS_CUDA(cudaMalloc(&c.pk_field, n * sizeof(float)), "cudaMalloc batch");
     PCS_CUDA(cudaMalloc(&c.pk_mask, n), "cudaMalloc batch");

@@ -149,7 +149,7 @@ extern "C" pcs_status pcs_solve_slices_noalloc(const float* field, const unsigne
         d.ready = true;
     }
     int ncl = 0, aux = 0;
-    const pcs::KernelEntry* entry = pcs::default_entry(H, W, 0, {S, true, 0}, &ncl, &aux, &e);
+    const pcs::KernelEntry* entry = pcs::default_entry(H, W, 0, {S, true, 0, 0, 0.0}, &ncl, &aux, &e);
     if (e != cudaSuccess) return err(PCS_ECUDA, "kernel attributes", e);
     int k_size = -1;
     for (int k = 0; k < kNumSizes; ++k)

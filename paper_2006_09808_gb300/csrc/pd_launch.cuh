@@ -205,6 +205,9 @@ struct ShapeCall {
     int S;       // slices
     bool whole;  // whole slices per cluster (no balanced schedule)
     int cap;     // pcs_options.max_clusters
+    // other solves on the device: how many, and their slices in units of this size's pixels
+    int solves;
+    double in_flight;
 };
 
 // The entry such a call runs (kernel: 0 the size's default, 1, 2 the option), how many of its clusters

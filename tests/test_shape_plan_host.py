@@ -57,6 +57,20 @@ def test_max_clusters_choices():
     assert plan(128, 64, max_clusters=8) == (4, 8)  # not 8 of the 2-CTA shape
 
 
+@pytest.mark.parametrize("H,alone,crowd", [(64, 4, 1), (128, 8, 2), (192, 12, 3), (256, 16, 4)])
+def test_solves_in_flight_shrink_the_clusters(H, alone, crowd):
+    """Alone, a slice takes the largest cluster; beside many others the shape with the least SM time."""
+    assert plan(H, 1)[0] == alone
+    assert plan(H, 1, in_flight=200.0)[0] == crowd
+    sizes = [plan(H, 1, in_flight=float(n))[0] for n in range(0, 200, 4)]
+    assert sizes == sorted(sizes, reverse=True)
+    assert plan(256, 1, solves=23, in_flight=23.0)[0] == 4  # 24 calls of one slice
+    assert plan(192, 1, solves=31, in_flight=31.0)[0] == 3
+    assert plan(192, 1, solves=35, in_flight=35.0)[0] == 6  # more streams than run at once: two solves in turn
+    with pytest.raises(pcs.PcsError):
+        plan(H, 1, in_flight=-1.0)
+
+
 def test_device_without_room_for_the_chosen_shapes():
     """A part of a GPU that holds no 16-CTA (or 8-CTA) cluster solves with a half-spectrum variant."""
     assert pcs.pcs_shape_plan(512, 512, 5, {16: 0, 8: 2}) == (8, 2)
