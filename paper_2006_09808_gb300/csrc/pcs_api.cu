@@ -98,7 +98,7 @@ cudaError_t prepared(const pcs::KernelEntry* e, int* mc, int* aux) {
 
 namespace pcs {
 
-// us per iteration of the call on mc resident clusters of the entry: the entry's time, times the rounds
+// us per iteration of the call on mc resident clusters of the entry: its time us, times the rounds
 // when the slices outnumber the clusters.  The balanced schedule makes fractions of a round count;
 // without it a cluster solves whole slices, and one slice more than the clusters costs a round (20
 // slices of 128 x 128 on 19 8-CTA clusters: 16.7 us per iteration, 9.3 on 4-CTA clusters).  Slices of
@@ -107,20 +107,20 @@ namespace pcs {
 // contexts of 256 x 256 on 24 streams: 49 us per iteration in 16-CTA clusters, 22.6 in 4-CTA ones).  The
 // device runs the streams of up to 32 of them at once; more wait for one another (36 streams take the
 // time of two solves in 3-CTA clusters at 192 x 192, 45 us, but 32 in larger ones).
-static double entry_cost(const KernelEntry& e, const ShapeCall& call, int mc) {
+static double entry_cost(float us, const ShapeCall& call, int mc) {
     constexpr int kStreams = 32;
     const double rounds = (double)call.S / mc;
     const double own = call.whole ? std::ceil(rounds) : std::max(1.0, rounds);
-    return e.us * std::max(own * (1 + call.solves / kStreams), (call.S + call.in_flight) / mc);
+    return us * std::max(own * (1 + call.solves / kStreams), (call.S + call.in_flight) / mc);
 }
 
-// Clusters of the entry that a call may use of `resident` ones: one CTA per SM, and with max_clusters
+// Clusters of the entry that a call may use of `resident` ones, per_sm CTAs per SM: with max_clusters
 // at most that many clusters on at most as many SMs as that many of the size's base clusters (aux_C
 // CTAs each).  A caller that leaves SMs to other work by it keeps them: one slice of 256 x 256 with
 // max_clusters = 1 runs on 4 SMs and not in a 16-CTA cluster.  The size's smallest shape rounds up to
 // whole clusters (192, 384 and 512: 3, 8 and 16 CTAs on a base of 2, 4 and 8).
-static int usable_clusters(const KernelEntry& e, bool smallest, int resident, int sms, int cap) {
-    const int mc = std::min(resident, sms / e.C);
+static int usable_clusters(const KernelEntry& e, bool smallest, int resident, int sms, int per_sm, int cap) {
+    const int mc = std::min(resident, per_sm * sms / e.C);
     if (cap <= 0) return mc;
     const long long sm = (long long)cap * e.aux_C;
     return (int)std::min<long long>({mc, cap, (sm + (smallest ? e.C - 1 : 0)) / e.C});
@@ -140,13 +140,15 @@ static const KernelEntry* cheapest_entry(int H, int W, int is_resident, const Sh
     double best_cost = 0.0;
     for (const auto& e : entries()) {
         if (!candidate(e)) continue;
-        const int mc = usable_clusters(e, e.C == least_C, resident(e), sms, call.cap);
-        if (mc < 1) continue;
-        const double cost = entry_cost(e, call, mc);
-        if (!best || cost < best_cost) {
-            best = &e;
-            best_cost = cost;
-            *max_clusters = mc;
+        for (int per_sm = 1; per_sm <= (e.us2 > 0.f ? 2 : 1); ++per_sm) {
+            const int mc = usable_clusters(e, e.C == least_C, resident(e), sms, per_sm, call.cap);
+            if (mc < 1) continue;
+            const double cost = entry_cost(per_sm == 1 ? e.us : e.us2, call, mc);
+            if (!best || cost < best_cost) {
+                best = &e;
+                best_cost = cost;
+                *max_clusters = mc;
+            }
         }
     }
     if (best) return best;
@@ -1110,7 +1112,8 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
                     mc = std::min(mc, call.cap);
                     best_mc = std::min(best_mc, call.cap);
                 }
-                if (mc < 1 || pcs::entry_cost(e, call, mc) > 1.5 * pcs::entry_cost(*best_known, call, std::max(1, best_mc)))
+                if (mc < 1 || pcs::entry_cost(e.us, call, mc) >
+                                  1.5 * pcs::entry_cost(best_known->us, call, std::max(1, best_mc)))
                     continue;
             }
         }

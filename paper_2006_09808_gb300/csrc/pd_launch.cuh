@@ -27,12 +27,13 @@ struct KernelEntry {
     // the balanced-schedule instantiation of the iteration kernel (NULL for pd_resident_kernel)
     cudaError_t (*launch_sched)(const PDParams& prm, int n_clusters, cudaStream_t stream);
     int aux_C;     // cluster size of the diagnostics and power iteration
-    // Measured us per iteration with at most one CTA per SM, all clusters at work (anisotropic and
+    // Measured us per iteration with all the clusters at work that SMs / C allows (anisotropic and
     // unweighted; by isotropic weighted times the choice would be the same or within 8%).  The entries
     // of a size that have it give bit-identical results, and contexts without variant options take the
     // cheapest for the call's slice count (default_entry in pcs_api.cu).  0: only by option or
     // autotuner.
     float us;
+    float us2;  // the same with twice as many, two CTAs per SM; 0: shared memory allows one
 };
 
 template <class G>
@@ -113,7 +114,7 @@ template <class G>
 constexpr KernelEntry make_entry() {
     return KernelEntry{G::H,           G::W,           G::C,       0,
                        G::SMEM_BYTES,  G::NT,          100 * G::ER + G::EC, &prepare_all<G>,
-                       &launch_pd<G>,  &launch_report<G>, &launch_opnorm<G>, &launch_pd_sched<G>, G::C, 0.f};
+                       &launch_pd<G>,  &launch_report<G>, &launch_opnorm<G>, &launch_pd_sched<G>, G::C, 0.f, 0.f};
 }
 
 // One-transform-pair variant (pd_pair.cuh), state on chip: it serves both kernel options (RES is the
@@ -139,11 +140,12 @@ cudaError_t prepare_pair(int* max_clusters, int* max_clusters_aux) {
     return cudaSuccess;
 }
 template <class GP, class G, int RES = 0>
-constexpr KernelEntry make_pair_entry(float us) {
+constexpr KernelEntry make_pair_entry(float us, float us2 = 0.f) {
     static_assert(GP::H == G::H && GP::W == G::W, "same slices");
     return KernelEntry{GP::H,           GP::W,          GP::C,       RES,
                        GP::SMEM_BYTES,  GP::NT,         100 * GP::E + GP::E, &prepare_pair<GP, G>,
-                       &launch_pair<GP>, &launch_report<G>, &launch_opnorm<G>, &launch_pair_sched<GP>, G::C, us};
+                       &launch_pair<GP>, &launch_report<G>, &launch_opnorm<G>, &launch_pair_sched<GP>, G::C,
+                       us,              us2};
 }
 
 // Resident variant: the iteration kernel keeps the state on chip; the
@@ -168,7 +170,7 @@ constexpr KernelEntry make_resident_entry() {
     using G = typename GR::B;
     return KernelEntry{GR::H,           GR::W,          GR::C,       1,
                        GR::SMEM_BYTES,  GR::NT,         100 * GR::ER + GR::EC, &prepare_res<GR>,
-                       &launch_res<GR>, &launch_report<G>, &launch_opnorm<G>, nullptr, G::C, 0.f};
+                       &launch_res<GR>, &launch_report<G>, &launch_opnorm<G>, nullptr, G::C, 0.f, 0.f};
 }
 
 // FP64 variant (precision study): iteration kernel only.
@@ -211,7 +213,7 @@ struct ShapeCall {
 };
 
 // The entry such a call runs (kernel: 0 the size's default, 1, 2 the option), how many of its clusters
-// are resident (one CTA per SM) and how many of the auxiliary kernels'.  The counts are kept per
+// it may use and how many of the auxiliary kernels'.  The counts are kept per
 // device; the attributes are set when a count is first taken and by every pcs_create.  NULL: none
 // compiled.
 const KernelEntry* default_entry(int H, int W, int kernel, const ShapeCall& call, int* max_clusters,

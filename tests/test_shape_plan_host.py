@@ -11,7 +11,7 @@ pytestmark = pytest.mark.skipif(shutil.which("nvcc") is None and not os.path.exi
                                 reason="needs nvcc or a built libpcs.so")
 
 # resident clusters by cluster size, as a 152-SM device reports them
-RESIDENT = {64: {4: 37, 2: 76, 1: 152}, 128: {8: 19, 4: 36, 2: 76, 1: 152}, 192: {12: 8, 6: 20, 3: 48},
+RESIDENT = {64: {4: 76, 2: 152, 1: 152}, 128: {8: 38, 4: 36, 2: 76, 1: 152}, 192: {12: 16, 6: 20, 3: 48},
             256: {16: 8, 8: 15, 4: 36}, 384: {8: 15}, 512: {16: 8}}
 
 
@@ -29,8 +29,8 @@ def plan(H, S, **query):
 @pytest.mark.parametrize("H,S,balanced,whole", [
     # one slice more than the larger clusters hold: a fraction of a round on the balanced schedule,
     # a whole round without it
-    (128, 19, 8, 8), (128, 20, 4, 4), (192, 8, 12, 12), (192, 9, 12, 6), (256, 8, 16, 16), (256, 9, 16, 8),
-    (256, 15, 8, 8), (256, 16, 8, 4), (256, 37, 4, 4),
+    (64, 38, 4, 4), (64, 39, 2, 2), (128, 19, 8, 8), (128, 20, 4, 4), (192, 16, 12, 12), (192, 17, 6, 6),
+    (192, 21, 6, 3), (256, 8, 16, 16), (256, 9, 16, 8), (256, 15, 8, 8), (256, 16, 8, 4), (256, 37, 4, 4),
 ])
 def test_whole_slices_cost_whole_rounds(H, S, balanced, whole):
     assert plan(H, S) == (balanced, min(S, RESIDENT[H][balanced]))
