@@ -380,15 +380,15 @@ typedef struct pcs_volume {
     float *chi_out;            /* device [S][H][W] */
 } pcs_volume;
 
-/* What the autotuner chose for one slice size, and what it measured. */
+/* The variant of one slice size's last solve, and what the autotuner measured at its first. */
 typedef struct pcs_tuning {
     int H, W;
-    int cluster_size, kernel, threads; /* the chosen variant (kernel: 1 streaming, 2 resident) */
+    int cluster_size, kernel, threads; /* the variant (kernel: 1 streaming, 2 resident) */
     int n_candidates;
     double L;                          /* ||K||_2 of the full-mask operator; tau = sigma = 1/L */
     double ns_per_voxel_iter[8];       /* trial time of each candidate, in registry order */
     int cand_cluster_size[8], cand_kernel[8], cand_threads[8];
-    int tile;                          /* the chosen variant's FFT tile shape (see pcs_options.tile) */
+    int tile;                          /* the variant's FFT tile shape (see pcs_options.tile) */
     int cand_tile[8];
     int pad;
 } pcs_tuning;
@@ -402,7 +402,9 @@ typedef struct pcs_tuning {
  * of the full-mask operator K (Sec. II.A pseudocode step 1), computed once per
  * size on the GPU.  autotune != 0: the first solve of a new slice size times
  * every compiled kernel variant of that size on that call's slice count
- * (a short trial) and keeps the fastest; otherwise the library default (or
+ * (a short trial) and keeps the fastest -- for calls of other counts too,
+ * unless it is one of the cluster shapes that give the same bits, of which such
+ * a call takes its own (pcs_shape_plan); otherwise the library default (or
  * the variant opt selects) is used.
  */
 PCS_API pcs_status pcs_batch_create(pcs_batch **out, const pcs_options *opt, int autotune, void *cuda_stream);

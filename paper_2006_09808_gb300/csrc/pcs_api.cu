@@ -1045,6 +1045,10 @@ struct pcs_batch {
         int capacity = 0;
         pcs_tuning tuning{};
         bool tuned = false;
+        // the tuned variant, for calls of tuned_S slices; where it is one of the shapes that give the same
+        // bits, calls of other counts take theirs (a context without variant options)
+        const pcs::KernelEntry* tuned_entry = nullptr;
+        int tuned_S = 0;
     };
     pcs_options opt{};
     int autotune = 0;
@@ -1158,8 +1162,13 @@ pcs_status tune_class(pcs_batch* b, pcs_batch::Class& c, int S, int trial_iters)
     cudaFree(m);
     if (st != PCS_OK) return st;
     c.tuned = true;
+    c.tuned_S = S;
+    c.tuned_entry = find_entry(t.H, t.W, t.cluster_size, t.kernel, t.threads, t.tile);
     return PCS_OK;
 }
+
+constexpr int kMostTrialSlices = 128;
+int trial_slices(int S) { return std::min(S, kMostTrialSlices); }
 
 // Make class c ready for S slices: variant chosen, context and packed buffers
 // large enough, L known.
@@ -1170,7 +1179,7 @@ pcs_status prepare_class(pcs_batch* b, pcs_batch::Class& c, int S) {
         PCS_CUDA(cudaEventCreateWithFlags(&c.solved, cudaEventDisableTiming), "cudaEventCreate");
     }
     if (b->autotune && !c.tuned) {
-        pcs_status st = tune_class(b, c, S < 128 ? S : 128, 40);
+        pcs_status st = tune_class(b, c, trial_slices(S), 40);
         if (st != PCS_OK) return st;
     }
     if (c.ctx && c.capacity >= S) return PCS_OK;
@@ -1186,7 +1195,10 @@ pcs_status prepare_class(pcs_batch* b, pcs_batch::Class& c, int S) {
     c.inv_den = nullptr;
     pcs_options o = b->opt;
     o.use_graph = 0;
-    if (c.tuned) {
+    if (c.tuned && c.tuned_entry && c.tuned_entry->us > 0.f) {
+        o.cluster_size = o.threads = o.tile = 0;
+        o.kernel = c.tuning.kernel;
+    } else if (c.tuned) {
         o.cluster_size = c.tuning.cluster_size;
         o.kernel = c.tuning.kernel;
         o.threads = c.tuning.threads;
@@ -1298,7 +1310,14 @@ pcs_status pcs_batch_solve(pcs_batch* b, const pcs_volume* vols, int n_vols, int
         }
         PCS_CUDA(cudaMemcpyAsync(C.inv_den, inv.data(), inv.size() * sizeof(float), cudaMemcpyHostToDevice, C.stream), "lambda upload");
         if (prev) PCS_CUDA(cudaStreamWaitEvent(C.stream, prev->solved, 0), "wait for the previous class");
-        pcs_status st = launch_solve(C.ctx, C.pk_field, C.pk_mask, cls_S[c], 1.0, tau, sigma, n_iter, C.pk_chi, C.inv_den);
+        const pcs::KernelEntry* entry = nullptr;
+        int ncl = 0, aux = 0;
+        if (C.ctx->by_count && C.tuned && trial_slices(cls_S[c]) == C.tuned_S) {
+            entry = C.tuned_entry;
+            PCS_CUDA(prepared(entry, &ncl, &aux), "kernel attributes");
+        }
+        pcs_status st = launch_solve(C.ctx, C.pk_field, C.pk_mask, cls_S[c], 1.0, tau, sigma, n_iter, C.pk_chi,
+                                     C.inv_den, entry, ncl);
         if (st != PCS_OK) return st;
         PCS_CUDA(cudaEventRecord(C.solved, C.stream), "solved record");
         prev = &C;
@@ -1319,20 +1338,16 @@ pcs_status pcs_batch_tuning(pcs_batch* b, int H, int W, pcs_tuning* out) {
     if (!b || !out) return fail(PCS_EINVAL, "NULL argument");
     for (const auto& c : b->classes)
         if (c.H == H && c.W == W) {
-            if (!c.tuned) {
-                const pcs::KernelEntry* e = c.ctx ? c.ctx->entry : find_entry(H, W, 0);
-                *out = pcs_tuning{};
-                out->H = H;
-                out->W = W;
-                out->cluster_size = e ? e->C : 0;
-                out->kernel = e ? (e->resident ? 2 : 1) : 0;
-                out->threads = e ? e->threads : 0;
-                out->tile = e ? e->tile : 0;
-                out->L = c.L;
-                return PCS_OK;
-            }
             *out = c.tuning;
+            out->H = H;
+            out->W = W;
             out->L = c.L;
+            // the variant of the size's last solve
+            const pcs::KernelEntry* e = c.ctx ? (c.ctx->ran_entry ? c.ctx->ran_entry : c.ctx->entry) : find_entry(H, W, 0);
+            out->cluster_size = e ? e->C : 0;
+            out->kernel = e ? (e->resident ? 2 : 1) : 0;
+            out->threads = e ? e->threads : 0;
+            out->tile = e ? e->tile : 0;
             return PCS_OK;
         }
     return fail(PCS_EINVAL, "size %d x %d not solved by this batch", H, W);
