@@ -24,7 +24,9 @@
 // reports it.
 // Step sizes are tau = sigma = 1/L(H, W) (Sec. II.A pseudocode step 1), L the
 // full-mask operator norm, computed once per slice size; the kernel variant
-// of each size is the one the batch autotuner picks.  The primal/dual state of
+// of each size is the one the batch autotuner picks or, where that is one of the
+// cluster shapes that give the same bits, the shape that suits the chunk and what
+// the other slots are at work on (default_entry).  The primal/dual state of
 // an admitted request stays in device memory until the request completes.
 #include <cuda_runtime.h>
 
@@ -289,6 +291,11 @@ pcs_status size_setup(pcs_server* sv, int H, int W, SizeInfo** out) {
     if (!si.entry || !(si.L > 0.0)) return pcs::set_last_error(PCS_ECUDA, "serve: size set-up");
     int aux = 0;
     if (si.entry->prepare(&si.max_clusters, &aux) != cudaSuccess) return pcs::set_last_error(PCS_ECUDA, "serve: prepare");
+    if (si.entry->us > 0.f) {  // the shapes a chunk may take: their attributes now, not in the loop
+        int ncl = 0;
+        if (!pcs::default_entry(H, W, si.tuning.kernel, {S, true, 0, 0, 0.0}, &ncl, &aux, &e) || e != cudaSuccess)
+            return pcs::set_last_error(PCS_ECUDA, "serve: prepare");
+    }
     std::vector<float> dtab, ddtab;
     std::vector<float2> tw;
     pcs::build_dipole_tables(H, W, sv->cfg.b0_axis, dtab, ddtab);
@@ -345,6 +352,30 @@ void admit(pcs_server* sv) {
     }
 }
 
+// The entry and clusters a chunk of n slices of request r runs on.  Tuned on 16 slices alone, the large
+// clusters of 192 x 192 and 256 x 256 cost up to twice the SM time of the small ones (144 against 67
+// SM-us per slice and iteration at 192 x 192), which a loaded server has no SMs to spare for.
+cudaError_t chunk_entry(const pcs_server* sv, const SizeInfo& si, const Request& r, int n, const pcs::KernelEntry** entry,
+                        int* clusters) {
+    *entry = si.entry;
+    *clusters = si.max_clusters;
+    if (si.entry->us > 0.f) {
+        pcs::ShapeCall call{n, true, 0, 0, 0.0};
+        for (const auto& kv : sv->reqs) {
+            const Request& o = kv.second;
+            if (o.id == r.id || o.chunks.empty()) continue;  // the slot's own chunks run in turn
+            ++call.solves;
+            call.in_flight += (double)o.chunks.front().n * o.H * o.W / ((double)r.H * r.W);
+        }
+        cudaError_t e = cudaSuccess;
+        int aux = 0;
+        *entry = pcs::default_entry(r.H, r.W, si.tuning.kernel, call, clusters, &aux, &e);
+        if (e != cudaSuccess) return e;
+    }
+    *clusters = std::max(1, std::min(*clusters, n));
+    return cudaSuccess;
+}
+
 // Launch every arrived slice range of admitted requests.  A request whose copy or launch fails
 // gets that status; its later slices are dropped.
 bool launch_arrived(pcs_server* sv) {
@@ -398,8 +429,10 @@ bool launch_arrived(pcs_server* sv) {
                 prm.tau = (float)(1.0 / si->L);
                 prm.inv_den = (float)(1.0 / (1.0 + (1.0 / si->L) / r.lambda));
                 prm.inv_den_slice = nullptr;
-                const int ncl = std::min(si->max_clusters, a.n);
-                e3 = si->entry->launch(prm, ncl < 1 ? 1 : ncl, sl.stream);
+                const pcs::KernelEntry* entry = nullptr;
+                int clusters = 0;
+                e3 = chunk_entry(sv, *si, r, a.n, &entry, &clusters);
+                if (e3 == cudaSuccess) e3 = entry->launch(prm, clusters, sl.stream);
             }
             if (r.fail_next) {  // injected on the host: this launch reports an error code
                 r.fail_next = false;
