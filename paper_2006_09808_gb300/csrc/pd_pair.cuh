@@ -473,10 +473,11 @@ struct StTmem {
         const int a = (G::P_GLOBAL && c.a > kP) ? c.a - 1 : c.a;
         return base + (unsigned)(2 * G::E * a + 4 * c.q);
     }
-    // the four arrays' chunk q, in the order q_x, q_y, chi, p
-    __device__ __forceinline__ void load_all(float4 (&v)[4], int q) const {
+    // the four arrays' chunk q, in the order q_x, q_y, chi, p.  with_p false: p is not used, and not read
+    // from global memory (chi of the last iteration is being written over it)
+    __device__ __forceinline__ void load_all(float4 (&v)[4], int q, bool with_p = true) const {
         if constexpr (G::P_GLOBAL) {
-            v[3] = __ldcg(gp + q * G::NT);
+            v[3] = with_p ? __ldcg(gp + q * G::NT) : make_float4(0.f, 0.f, 0.f, 0.f);
             float4 t[3];
             load(t, {{kQx, q}, {kQy, q}, {kChi, q}});
             v[0] = t[0], v[1] = t[1], v[2] = t[2];
@@ -532,7 +533,7 @@ struct StShared {
     __device__ __forceinline__ void init(unsigned, float* mem) {
         base = reinterpret_cast<float4*>(mem) + threadIdx.x;
     }
-    __device__ __forceinline__ void load_all(float4 (&v)[4], int q) const {
+    __device__ __forceinline__ void load_all(float4 (&v)[4], int q, bool = true) const {
         load(v, {{kQx, q}, {kQy, q}, {kChi, q}, {kP, q}});
     }
     template <int K>
@@ -901,7 +902,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
 #pragma unroll
                     for (int q = 0; q < NCH; ++q) {
                         float4 v[4];
-                        cx.st.load_all(v, q);
+                        cx.st.load_all(v, q, !last);
                         const float2 qu = G::SLOT_GLOBAL ? u0 : slot.ld_up(q);  // q_y of the row above row a
                         u0 = u1;
                         if (G::SLOT_GLOBAL && q + 2 < NCH) u1 = slot.ld_up(q + 2);
