@@ -57,6 +57,18 @@ bool gen_plan(int n, GenPlan* pl) {
     return true;
 }
 
+// The roots of unity of a plan, then the coefficients of its direct stages (gen_fill_tables).
+void gen_tables(GenPlan* pl, std::vector<float2>* tab) {
+    pcs::build_twiddles(pl->n, *tab);
+    pl->ncoef = 0;
+    for (int st = 0; st < pl->nst; ++st) {
+        const int r = pl->r[st];
+        if (r < 5 || r == 6) continue;
+        for (int m = 0; m < r; ++m) tab->push_back((*tab)[(size_t)m * (pl->n / r)]);
+        pl->ncoef += r;
+    }
+}
+
 pcs_status failg(pcs_status st, const char* what, cudaError_t e = cudaSuccess) {
     char buf[256];
     if (e != cudaSuccess) {
@@ -83,8 +95,8 @@ constexpr ColEntry col_entry() {
 const ColEntry k_cols[] = {col_entry<64>(),  col_entry<128>(), col_entry<192>(),
                            col_entry<256>(), col_entry<384>(), col_entry<512>()};
 
-size_t rows_smem(int W) { return sizeof(float2) * (size_t)W * (1 + 2 * pcs::kGenRowWarps); }
-size_t cols_smem(int H) { return sizeof(float2) * ((size_t)H + (size_t)(2 * H + 1) * pcs::kGenColTile); }
+size_t rows_smem(int W) { return sizeof(float2) * ((size_t)W * (1 + 2 * pcs::kGenRowWarps) + pcs::kGenCoef); }
+size_t cols_smem(int H) { return sizeof(float2) * ((size_t)H + pcs::kGenCoef + (size_t)(2 * H + 1) * pcs::kGenColTile); }
 
 bool gen_shape_ok(int H, int W, GenPlan* prow, GenPlan* pcol) {
     return H % 2 == 0 && W % 2 == 0 && gen_plan(W, prow) && gen_plan(H, pcol);
@@ -158,21 +170,24 @@ cudaError_t gen_create(GenSolver** out, int H, int W, int max_slices, int b0_axi
     gs->scols = ce ? ce->smem : cols_smem(H);
     gs->max_slices = max_slices;
     std::vector<float2> tw_r, tw_c;
-    build_twiddles(W, tw_r);
-    build_twiddles(H, tw_c);
+    gen_tables(&gs->g.prow, &tw_r);
+    gen_tables(&gs->g.pcol, &tw_c);
     // the dynamic shared-memory limit is a per-function attribute shared by every size: set it
     // to what the largest accepted size needs, so that solvers of several sizes coexist
     const int rows_max = (int)rows_smem(kGenMaxLen), cols_max = (int)cols_smem(kGenMaxLen);
     cudaError_t e;
-    if ((e = cudaMalloc(&gs->tabs, (size_t)(W + H) * sizeof(float2))) != cudaSuccess ||
+    if ((e = cudaMalloc(&gs->tabs, (tw_r.size() + tw_c.size()) * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&gs->spec, (size_t)max_slices * H * M1 * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&gs->partial, (size_t)max_slices * (H / 2) * kGenReportSums * sizeof(double))) !=
             cudaSuccess ||
-        (e = cudaMemcpy(gs->tabs, tw_r.data(), W * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(gs->tabs + W, tw_c.data(), H * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(gen_rows_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(gen_rows_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
+        (e = cudaMemcpy(gs->tabs, tw_r.data(), tw_r.size() * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(gs->tabs + tw_r.size(), tw_c.data(), tw_c.size() * sizeof(float2),
+                        cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(gen_rows_kernel<32, kGenRowCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  rows_max)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(gen_rows_kernel<64, kGenRowCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  rows_max)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(gen_rows_kernel<64, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
             cudaSuccess ||
         (e = cudaFuncSetAttribute(gen_report_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
             cudaSuccess ||
@@ -186,7 +201,7 @@ cudaError_t gen_create(GenSolver** out, int H, int W, int max_slices, int b0_axi
     GenParams& g = gs->g;
     g.spec = gs->spec;
     g.trow = gs->tabs;
-    g.tcol = gs->tabs + W;
+    g.tcol = gs->tabs + tw_r.size();
     g.H = H;
     g.W = W;
     g.M1 = M1;
@@ -252,11 +267,14 @@ cudaError_t gen_enqueue(GenSolver* gs, const float* field, const unsigned char* 
     // two warps per row pair (200 iterations, one / two warps, ms): 12 slices of 128x132 5.82 / 5.30, 9 of
     // 90x170 9.07 / 7.33, 25 of 256x258 14.2 / 13.4; but 42 of 128x132 7.55 / 9.01: not for short rows
     // that already fill the GPU (three 8-warp CTAs on each of 152 SMs)
-    const bool two = g.W >= 192 || 2 * pairs <= 152 * 3 * kGenRowWarps;
-    auto rows = two ? &gen_rows_kernel<64> : &gen_rows_kernel<32>;
+    const bool few = 2 * pairs <= 152 * 3 * kGenRowWarps;
+    const bool two = g.W >= 192 || few;
+    auto rows = !two  ? &gen_rows_kernel<32, kGenRowCtas>
+                : few ? &gen_rows_kernel<64, 3>
+                      : &gen_rows_kernel<64, kGenRowCtas>;
     const int per_cta = kGenRowWarps / (two ? 2 : 1);
     const dim3 grid_l((pairs + per_cta - 1) / per_cta);
-    const size_t smem_l = sizeof(float2) * (size_t)g.W * (1 + 2 * per_cta);
+    const size_t smem_l = sizeof(float2) * ((size_t)g.W * (1 + 2 * per_cta) + kGenCoef);
     for (int it = 0; it < n_iter; ++it) {
         g.phase = 0;
         g.store = 1;

@@ -5,7 +5,7 @@
 //
 // Per half step two launches, the half spectrum [S][H][W/2 + 1] (row-major,
 // complex) held in global memory between them:
-//   row kernel:    one warp per pair of rows; the two real rows travel as one
+//   row kernel:    one or two warps per pair of rows; the two real rows travel as one
 //                  complex row (a + i b) through a length-W DFT in shared memory
 //                  -> the dual or primal row phase -> forward DFT, split back into
 //                  the two half-spectrum rows
@@ -13,8 +13,8 @@
 //                  fft_core.cuh for H in {64, 128, 192, 256, 384, 512} (pencils
 //                  of lanes, gen_cols_fft_kernel), else one warp per spectrum
 //                  column with the shared-memory DFT (gen_cols_kernel)
-// The shared-memory DFTs are mixed-radix Stockham passes: 2, 3, 4 as butterflies,
-// larger odd primes as a symmetric direct DFT (terms q and r - q paired).
+// The shared-memory DFTs are mixed-radix Stockham passes: 2, 3, 4, 6 as butterflies,
+// larger primes as a symmetric direct DFT (terms q and r - q paired).
 // Also here: the FP64 report kernel and the power iteration for ||K||, which reuse
 // the row transforms and the column pass.
 #pragma once
@@ -27,11 +27,17 @@ namespace pcs {
 
 constexpr int kGenMaxStages = 12;
 constexpr int kGenRowWarps = 8;   // row pairs per CTA of the row, report and power-iteration kernels
+// CTAs per SM that the row kernels' registers are set for.  Left to itself the compiler took 80, three
+// CTAs, and solves of more row pairs than those hold took a second wave: 72 slices of 128 x 132, one
+// warp per pair, 56.6 us per iteration, 45.9 with four.
+constexpr int kGenRowCtas = 4;
 constexpr int kGenColTile = 16;   // spectrum columns per CTA of the shared-memory column kernel
+constexpr int kGenCoef = 64;      // coefficients of the direct stages: the primes >= 5 of a length add up to at most 61
 
 struct GenPlan {
     int n;                  // transform length
     int nst;                // number of stages
+    int ncoef;              // coefficients of the direct stages
     int r[kGenMaxStages];   // radices, product n
 };
 
@@ -45,8 +51,8 @@ struct GenParams {
     float* qx;
     float* qy;
     float2* spec;          // [S][H][M1]
-    const float2* trow;    // exp(-2 pi i n / W), n < W
-    const float2* tcol;    // exp(-2 pi i n / H), n < H
+    const float2* trow;    // tables of prow: exp(-2 pi i n / W), n < W, then the coefficients
+    const float2* tcol;    // tables of pcol
     GenPlan prow, pcol;
     int S, H, W, M1;       // M1 = W / 2 + 1
     float sigma, tau, inv_den;
@@ -84,14 +90,23 @@ __device__ __forceinline__ void fma_pair(float2& acc, float2 v, float c) {
     acc = __ffma2_rn(v, make_float2(c, c), acc);
 }
 
+// Tables of a transform, to shared memory (whole CTA; the caller's barrier follows): its n roots of unity,
+// then the r coefficients (cos, -sin) of 2 pi m / r of each direct stage side by side (gen_tables on the
+// host).  Read from the roots, they lie n / r entries apart: with n / r = 16 the lanes of a stage share
+// one bank (28 slices of 128 x 464 = 16 x 29, one warp per pair: 90.5 us per iteration, 68.7 side by side).
+__device__ __forceinline__ void gen_fill_tables(float2* T, const float2* __restrict__ tab, const GenPlan& pl) {
+    for (int t = threadIdx.x; t < pl.n + pl.ncoef; t += blockDim.x) T[t] = tab[t];
+}
+
 // Direct part of a prime stage: outputs q' = qp and r - qp of NJ butterflies j = j0, j0 + dj, ...
 // (qp = 0: the plain sum), from the sums and differences sd[(q - 1) R + j] = (s_q, d_q) and v0[j]:
 // A = v_0 + sum s_q cos(2 pi m / r), B = sum d_q (-sin(2 pi m / r)), m = q qp mod r.  One coefficient
 // serves NJ butterflies, and the lanes that share them read the same (s, d): 2 NJ packed FMAs per
 // 1 + NJ loads (one lane per output and butterfly took 4 scalar FMAs per 3 loads).
-// A16: sd is 16-byte aligned.
-template <int NJ, bool A16>
-__device__ __forceinline__ void prime_outputs(const float2* sd, const float2* v0, float2* out, const float2* T, int r,
+// A16: sd is 16-byte aligned.  U: two terms at a time for up to U butterflies (more would not fit the
+// 64 registers of the four-CTA kernels).
+template <int NJ, int U, bool A16>
+__device__ __forceinline__ void prime_outputs(const float2* sd, const float2* v0, float2* out, const float2* P, int r,
                                               int R, int Ns, float invNs, int qp, int j0, int dj, float sg) {
     float2 A[NJ], B[NJ];
     int jj[NJ];
@@ -103,11 +118,12 @@ __device__ __forceinline__ void prime_outputs(const float2* sd, const float2* v0
     }
     const int h = (r - 1) / 2;
     int m = 0;
-#pragma unroll 2
+    constexpr int kUnroll = NJ <= U ? 2 : 1;
+#pragma unroll kUnroll
     for (int q = 1; q <= h; ++q) {
         m += qp;
         if (m >= r) m -= r;
-        const float2 c = T[m * R];  // (cos, -sin) of 2 pi m / r
+        const float2 c = P[m];  // (cos, -sin) of 2 pi m / r
         const float2* row = sd + 2 * (q - 1) * R;
 #pragma unroll
         for (int i = 0; i < NJ; ++i) {
@@ -143,12 +159,13 @@ __device__ __forceinline__ void prime_outputs(const float2* sd, const float2* v0
 // radix r after the radices so far multiply to Ns (R = n / r):
 //   X_out[(j / Ns) Ns r + k + q' Ns] = sum_q X_in[j + q R] w^(k q n/(Ns r)) w^(q q' R),
 // k = j mod Ns, w = exp(-+2 pi i / n), for j < R, q' < r.
-// A16: a and b are 16-byte aligned.
+// T: gen_fill_tables.  A16: a and b are 16-byte aligned.
 template <int LP = 32, bool A16 = true>
 __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan& pl, bool inv, int lane, int id = 0) {
     const int N = pl.n;
     const float sg = inv ? -1.f : 1.f;  // sign applied to the imaginary part of the forward twiddles
     auto tw = [T, sg](int i) { return make_float2(T[i].x, sg * T[i].y); };
+    const float2* P = T + N;
     int Ns = 1;
 #pragma unroll 1
     for (int st = 0; st < pl.nst; ++st) {
@@ -256,19 +273,23 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
             // lanes: h + 1 outputs, as many groups of butterflies as fit (r <= 61: at least one)
             const int nq = h + 1, jg = LP / nq, qp = lane % nq, g0 = lane / nq;
             const int per = (R + jg - 1) / jg;  // butterflies per lane
+            constexpr int U = LP == 32 ? 2 : 3;
+            // six at once as 3 + 3, not 4 + 4 with two of them idle
             if (g0 < jg) {
                 if (per <= 1) {
-                    prime_outputs<1, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, g0, jg, sg);
+                    prime_outputs<1, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, g0, jg, sg);
                 } else if (per == 2) {
-                    prime_outputs<2, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, g0, jg, sg);
-                } else if (per == 3) {
-                    prime_outputs<3, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, g0, jg, sg);
+                    prime_outputs<2, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, g0, jg, sg);
+                } else if (per % 3 == 0 || per == 5) {
+#pragma unroll 1
+                    for (int j = g0; j < R; j += 3 * jg) prime_outputs<3, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, j, jg, sg);
                 } else {
 #pragma unroll 1
-                    for (int j = g0; j < R; j += 4 * jg) prime_outputs<4, A16>(sd, v0, a, T, r, R, Ns, invNs, qp, j, jg, sg);
+                    for (int j = g0; j < R; j += 4 * jg) prime_outputs<4, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, j, jg, sg);
                 }
             }
             lanes_sync<LP>(id);
+            P += r;
             Ns *= r;
             continue;  // result in a: no swap
         }
@@ -284,20 +305,21 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
 // Row kernel: LP lanes (one or two warps) take rows i0 = 2 pr, i1 = i0 + 1 of one slice.  The kernel is
 // bound by latency (25 slices of 256 x 258: half of the issue slots used by 21 warps per SM), which a
 // second warp per pair shortens; where the pairs fill the GPU with one warp each and the row is short,
-// the second only adds idle lanes (host rule in gen_enqueue).
-template <int LP>
-__global__ void __launch_bounds__(kGenRowWarps * 32) gen_rows_kernel(GenParams g) {
+// the second only adds idle lanes (host rule in gen_enqueue).  CTAS: CTAs per SM (kGenRowCtas, or three
+// where those hold every pair: 80 registers are up to 3% quicker then).
+template <int LP, int CTAS>
+__global__ void __launch_bounds__(kGenRowWarps * 32, CTAS) gen_rows_kernel(GenParams g) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int H = g.H, W = g.W, M1 = g.M1;
     float2* T = reinterpret_cast<float2*>(smem_raw);
-    for (int t = threadIdx.x; t < W; t += blockDim.x) T[t] = g.trow[t];
+    gen_fill_tables(T, g.trow, g.prow);
     __syncthreads();
     grid_dependency_wait();  // the previous launch's spectrum and state complete
     constexpr int PAIRS = kGenRowWarps * 32 / LP;  // row pairs per CTA
     const int lane = threadIdx.x % LP, wl = threadIdx.x & 31, grp = threadIdx.x / LP, bar = 1 + grp;
     const int pair = blockIdx.x * PAIRS + grp;
     if (pair >= g.S * (H / 2)) return;  // whole groups; no CTA barrier below
-    float2* bufa = T + W + (size_t)grp * 2 * W;
+    float2* bufa = T + W + kGenCoef + (size_t)grp * 2 * W;
     float2* bufb = bufa + W;
     const int s = pair / (H / 2);
     if (g.active && !g.active[s]) return;  // frozen slice (monitored solves): state kept as is
@@ -493,17 +515,17 @@ __device__ __forceinline__ void gen_store_rows(float2* o, float2* scratch, const
     }
 }
 
-__global__ void __launch_bounds__(kGenRowWarps * 32) gen_report_kernel(GenParams g, double* partial, double lam,
-                                                                        int mode) {
+__global__ void __launch_bounds__(kGenRowWarps * 32, kGenRowCtas)
+    gen_report_kernel(GenParams g, double* partial, double lam, int mode) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int H = g.H, W = g.W, M1 = g.M1;
     float2* T = reinterpret_cast<float2*>(smem_raw);
-    for (int t = threadIdx.x; t < W; t += blockDim.x) T[t] = g.trow[t];
+    gen_fill_tables(T, g.trow, g.prow);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int pair = blockIdx.x * kGenRowWarps + warp;
     if (pair >= g.S * (H / 2)) return;  // whole warps; no CTA barrier below
-    float2* bufa = T + W + (size_t)warp * 2 * W;
+    float2* bufa = T + W + kGenCoef + (size_t)warp * 2 * W;
     float2* bufb = bufa + W;
     const int s = pair / (H / 2);
     const int i0 = 2 * (pair - s * (H / 2)), i1 = i0 + 1;
@@ -626,18 +648,17 @@ __global__ void gen_opnorm_norm_kernel(const double* partial, int pairs_per_slic
     scale[s] = (yy > 0.0) ? (float)(1.0 / sqrt(yy)) : 0.f;
 }
 
-__global__ void __launch_bounds__(kGenRowWarps * 32) gen_opnorm_rows_kernel(GenParams g, const float* x, float* y,
-                                                                             const float* scale, double* partial,
-                                                                             int mode) {
+__global__ void __launch_bounds__(kGenRowWarps * 32, kGenRowCtas)
+    gen_opnorm_rows_kernel(GenParams g, const float* x, float* y, const float* scale, double* partial, int mode) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int H = g.H, W = g.W, M1 = g.M1;
     float2* T = reinterpret_cast<float2*>(smem_raw);
-    for (int t = threadIdx.x; t < W; t += blockDim.x) T[t] = g.trow[t];
+    gen_fill_tables(T, g.trow, g.prow);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int pair = blockIdx.x * kGenRowWarps + warp;
     if (pair >= g.S * (H / 2)) return;  // whole warps; no CTA barrier below
-    float2* bufa = T + W + (size_t)warp * 2 * W;
+    float2* bufa = T + W + kGenCoef + (size_t)warp * 2 * W;
     float2* bufb = bufa + W;
     const int s = pair / (H / 2);
     const int i0 = 2 * (pair - s * (H / 2)), i1 = i0 + 1;
@@ -722,11 +743,11 @@ __global__ void __launch_bounds__(kGenColTile * 32) gen_cols_kernel(GenParams g)
     const int H = g.H, W = g.W, M1 = g.M1;
     const int CS = 2 * H + 1;
     float2* T = reinterpret_cast<float2*>(smem_raw);
-    float2* cols = T + H;  // [kGenColTile][CS]
+    float2* cols = T + H + kGenCoef;  // [kGenColTile][CS]
     const int kx0 = blockIdx.x * kGenColTile, s = blockIdx.y;
     const int ncol = min(kGenColTile, M1 - kx0);
     float2* spec = g.spec + (size_t)s * H * M1;
-    for (int t = threadIdx.x; t < H; t += blockDim.x) T[t] = g.tcol[t];
+    gen_fill_tables(T, g.tcol, g.pcol);
     grid_dependency_wait();  // the previous launch's spectrum complete
     // rows of the tile: adjacent threads take adjacent columns
     const int c = threadIdx.x % kGenColTile;
