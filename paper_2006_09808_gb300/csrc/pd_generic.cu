@@ -63,7 +63,7 @@ void gen_tables(GenPlan* pl, std::vector<float2>* tab) {
     pl->ncoef = 0;
     for (int st = 0; st < pl->nst; ++st) {
         const int r = pl->r[st];
-        if (r < 5 || r == 6) continue;
+        if (r < 7) continue;
         for (int m = 0; m < r; ++m) tab->push_back((*tab)[(size_t)m * (pl->n / r)]);
         pl->ncoef += r;
     }

@@ -13,7 +13,7 @@
 //                  fft_core.cuh for H in {64, 128, 192, 256, 384, 512} (pencils
 //                  of lanes, gen_cols_fft_kernel), else one warp per spectrum
 //                  column with the shared-memory DFT (gen_cols_kernel)
-// The shared-memory DFTs are mixed-radix Stockham passes: 2, 3, 4, 6 as butterflies,
+// The shared-memory DFTs are mixed-radix Stockham passes: 2, 3, 4, 5, 6 as butterflies,
 // larger primes as a symmetric direct DFT (terms q and r - q paired).
 // Also here: the FP64 report kernel and the power iteration for ||K||, which reuse
 // the row transforms and the column pass.
@@ -32,7 +32,7 @@ constexpr int kGenRowWarps = 8;   // row pairs per CTA of the row, report and po
 // warp per pair, 56.6 us per iteration, 45.9 with four.
 constexpr int kGenRowCtas = 4;
 constexpr int kGenColTile = 16;   // spectrum columns per CTA of the shared-memory column kernel
-constexpr int kGenCoef = 64;      // coefficients of the direct stages: the primes >= 5 of a length add up to at most 61
+constexpr int kGenCoef = 64;      // coefficients of the direct stages: the primes >= 7 of a length add up to at most 61
 
 struct GenPlan {
     int n;                  // transform length
@@ -243,8 +243,39 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
                     put(5, v[4], v[1], -1.f);
                 }
             }
+        } else if (r == 5) {
+            // in registers, one lane per butterfly: a third of the barriers and half of the shared-memory
+            // traffic of the direct stage below (48 slices of 128 x 160, one warp per pair: 42.3 us
+            // per iteration, 36.5 so; 48 of 128 x 500: 131 and 89)
+            const float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;  // cos(2 pi / 5), cos(4 pi / 5)
+            const float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;   // sin(2 pi / 5), sin(4 pi / 5)
+#pragma unroll 1
+            for (int j = lane; j < R; j += LP) {
+                const int k = j - qdiv(j, invNs) * Ns;
+                float2 v[5];
+                v[0] = a[j];
+#pragma unroll
+                for (int q = 1; q < 5; ++q) v[q] = gcmul(a[j + q * R], tw(q * k * step));
+                auto add = [](float2 x, float2 y, float s) { return make_float2(x.x + s * y.x, x.y + s * y.y); };
+                const float2 p1 = add(v[1], v[4], 1.f), m1 = add(v[1], v[4], -1.f);
+                const float2 p2 = add(v[2], v[3], 1.f), m2 = add(v[2], v[3], -1.f);
+                // a + x p + y q
+                auto sum = [](float2 a, float x, float2 p, float y, float2 q) {
+                    return make_float2(fmaf(y, q.x, fmaf(x, p.x, a.x)), fmaf(y, q.y, fmaf(x, p.y, a.y)));
+                };
+                const float2 zero = make_float2(0.f, 0.f);
+                const float2 A1 = sum(v[0], c1, p1, c2, p2), A2 = sum(v[0], c2, p1, c1, p2);
+                const float2 B1 = sum(zero, s1, m1, s2, m2), B2 = sum(zero, s2, m1, -s1, m2);
+                float2* o = b + (j - k) * 5 + k;
+                // A -+ i B (forward)
+                o[0] = add(add(v[0], p1, 1.f), p2, 1.f);
+                o[Ns] = make_float2(A1.x + sg * B1.y, A1.y - sg * B1.x);
+                o[2 * Ns] = make_float2(A2.x + sg * B2.y, A2.y - sg * B2.x);
+                o[3 * Ns] = make_float2(A2.x - sg * B2.y, A2.y + sg * B2.x);
+                o[4 * Ns] = make_float2(A1.x - sg * B1.y, A1.y + sg * B1.x);
+            }
         } else {
-            // odd prime r >= 5: (1) pre-twiddle in place (not in the first stage: k = 0); (2) sums
+            // odd prime r >= 7: (1) pre-twiddle in place (not in the first stage: k = 0); (2) sums
             // s_q = v_q + v_(r-q) and differences d_q = v_q - v_(r-q) into b, side by side; (3) the
             // outputs q' and r - q' together (prime_outputs).  The result lands in a.
             if (Ns > 1) {
