@@ -116,6 +116,7 @@ struct GenSolver {
     void (*cols_kern)(GenParams) = nullptr;
     int col_tile = 0, col_threads = 0;
     size_t srows = 0, scols = 0;
+    int sms = 0;
 };
 
 bool gen_supported(int H, int W) {
@@ -176,7 +177,10 @@ cudaError_t gen_create(GenSolver** out, int H, int W, int max_slices, int b0_axi
     // to what the largest accepted size needs, so that solvers of several sizes coexist
     const int rows_max = (int)rows_smem(kGenMaxLen), cols_max = (int)cols_smem(kGenMaxLen);
     cudaError_t e;
-    if ((e = cudaMalloc(&gs->tabs, (tw_r.size() + tw_c.size()) * sizeof(float2))) != cudaSuccess ||
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&gs->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaMalloc(&gs->tabs, (tw_r.size() + tw_c.size()) * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&gs->spec, (size_t)max_slices * H * M1 * sizeof(float2))) != cudaSuccess ||
         (e = cudaMalloc(&gs->partial, (size_t)max_slices * (H / 2) * kGenReportSums * sizeof(double))) !=
             cudaSuccess ||
@@ -264,14 +268,21 @@ cudaError_t gen_enqueue(GenSolver* gs, const float* field, const unsigned char* 
     // that grid (37.8 against 42.6 ms per 256x258x25 solve).  The first launch follows the
     // caller's own stream work and is serialised.
     const dim3 blk_r(kGenRowWarps * 32), blk_c(gs->col_threads);
-    // two warps per row pair (200 iterations, one / two warps, ms): 12 slices of 128x132 5.82 / 5.30, 9 of
-    // 90x170 9.07 / 7.33, 25 of 256x258 14.2 / 13.4; but 42 of 128x132 7.55 / 9.01: not for short rows
-    // that already fill the GPU (three 8-warp CTAs on each of 152 SMs)
-    const bool few = 2 * pairs <= 152 * 3 * kGenRowWarps;
-    const bool two = g.W >= 192 || few;
-    auto rows = !two  ? &gen_rows_kernel<32, kGenRowCtas>
-                : few ? &gen_rows_kernel<64, 3>
-                      : &gen_rows_kernel<64, kGenRowCtas>;
+    // Two warps per row pair shorten its chain as long as both fit on the GPU at once (H = 128, us per
+    // iteration, one / two warps: 12 slices of W = 132 29.5 / 26.5, of 258 45 / 33.0; 28 of 132 33.1 / 30.6,
+    // of 258 50.9 / 39.8).  A fourth CTA per SM of them pays for the longer rows only (36 slices of 132
+    // 34.4 / 36.8, of 196 44.3 / 44.2, of 258 52.7 / 47.9), and beyond that wave a single warp is quicker
+    // (48 slices of 132 39 / 49, of 258 62 / 67, of 330 60 / 66), but for two exceptions: rows of 256 on just
+    // beyond the wave of single warps (84 slices of 132 59 / 67, of 258 101 / 96, of 330 110 / 106), and the
+    // longest rows, from W = 418 on with three of the one-warp CTAs in shared memory and not four (72
+    // slices of 372 97 / 98, of 464 178 / 131).
+    const int slots = gs->sms * kGenRowWarps;  // warps of one CTA on every SM
+    const bool wave = pairs <= kGenRowCtas * slots;
+    const bool two = 2 * pairs <= 3 * slots || (g.W >= 192 && 2 * pairs <= kGenRowCtas * slots) ||
+                     (g.W >= 256 && !wave && 2 * pairs <= 11 * slots) || g.W > 360;
+    auto rows = !two                     ? &gen_rows_kernel<32, kGenRowCtas>
+                : 2 * pairs <= 3 * slots ? &gen_rows_kernel<64, 3>
+                                         : &gen_rows_kernel<64, kGenRowCtas>;
     const int per_cta = kGenRowWarps / (two ? 2 : 1);
     const dim3 grid_l((pairs + per_cta - 1) / per_cta);
     const size_t smem_l = sizeof(float2) * ((size_t)g.W * (1 + 2 * per_cta) + kGenCoef);
