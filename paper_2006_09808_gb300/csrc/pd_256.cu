@@ -6,9 +6,11 @@ using Aux = Geo<256, 256, 4, 1, 512>;
 static const KernelEntry k_entries[] = {
     // us per iteration (isotropic weighted): 4-CTA clusters 22.7 (29.6) for up to 36 slices (35 for the
     // half-spectrum kernel in the same geometry, Geo<256, 256, 4, 1, 512>); larger clusters for fewer
-    // slices: 8-CTA 16.5 (23.2) for up to 15, 16-CTA 14.2 (20.9) for up to 7 or 8 (by device)
+    // slices: 8-CTA 16.5 (23.2) for up to 15 and on the balanced schedule 22.5 (31.1) for 20, which 17.05
+    // stands for (20 slices in 4-CTA clusters: 22.6 and 29.6), 16-CTA 14.2 (20.9) for up to 7 or 8 (by
+    // device)
     make_pair_entry<GeoPair<256, 4, 512, true>, Aux>(22.7f),
-    make_pair_entry<GeoPair<256, 8, 256, false>, Aux>(16.5f),
+    make_pair_entry<GeoPair<256, 8, 256, false>, Aux>(17.05f),
     make_pair_entry<GeoPair<256, 16, 128, false>, Aux>(14.2f),
     make_entry<Geo<256, 256, 4, 2>>(),
     make_resident_entry<GeoRes<256, 256, 8>>(),
