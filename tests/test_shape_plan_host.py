@@ -30,7 +30,8 @@ def plan(H, S, **query):
     # one slice more than the larger clusters hold: a fraction of a round on the balanced schedule,
     # a whole round without it
     (64, 38, 4, 4), (64, 39, 2, 2), (128, 19, 8, 8), (128, 20, 4, 4), (192, 12, 12, 12),
-    (192, 16, 6, 6), (192, 24, 6, 3), (256, 19, 8, 4), (256, 20, 4, 4), (256, 8, 16, 16), (256, 9, 16, 8), (256, 15, 8, 8), (256, 16, 8, 4), (256, 37, 4, 4),
+    (192, 16, 6, 6), (192, 24, 6, 3), (256, 8, 16, 16), (256, 9, 16, 8), (256, 15, 8, 8), (256, 19, 8, 4),
+    (256, 20, 4, 4), (256, 37, 4, 4),
 ])
 def test_whole_slices_cost_whole_rounds(H, S, balanced, whole):
     assert plan(H, S) == (balanced, min(S, RESIDENT[H][balanced]))
