@@ -66,13 +66,18 @@ typedef enum pcs_status {
 
 typedef struct pcs_options {
     int b0_axis;       /* 0 = B0 along rows / y (default), 1 = along columns / x */
-    int cluster_size;  /* 0 = library default for the slice size; else CTAs per slice (1,2,4,8,16) */
+    int cluster_size;  /* 0 = library default for the call (see pcs_shape_plan); else CTAs per slice of a
+                          compiled variant (1, 2, 4, 8 or 16; 2, 3, 6 or 12 at 192x192) */
     int max_clusters;  /* 0 = as many concurrent clusters as fit; else an upper bound.  Where the library
                           chooses the cluster size it also bounds the SMs, to max_clusters times 1 (64x64),
                           2 (192x192), 4 (128x128, 256x256, 384x384) or 8 (512x512), rounded up to a
                           cluster of the size's smallest shape */
-    int kernel;        /* 0 = library default; 1 = streaming (state in global memory);
-                          2 = resident (state kept on chip for all iterations) */
+    int kernel;        /* 0 = library default; 1 = a kernel that also solves weighted and resumes;
+                          2 = a kernel that keeps the state on chip for all iterations.  Where the
+                          cluster size is left to the library both run the one-pair kernel (state on
+                          chip) at 64x64 and 128x128, and so does 1 at the other sizes; the
+                          half-spectrum kernels (state in global memory, or resident) are reached by
+                          cluster_size, threads and tile */
     int threads;       /* 0 = library default; else threads per CTA of a compiled variant */
     int use_graph;     /* 1 = launch each solve as a CUDA graph, captured once per distinct argument
                           set and replayed (needs a non-NULL stream); 0 = direct launch */
@@ -204,7 +209,10 @@ PCS_API pcs_status pcs_schedule_plan(int S, int n_iter, int clusters, int *segme
 /*
  * The cluster shape a call without variant options takes for a compiled size: of the shapes that
  * give the same bits, the one whose measured time per iteration, times the rounds of its resident
- * clusters, is least.  cluster_sizes[k], resident[k] (n of them): the clusters of each size the
+ * clusters, is least.  (128x128 has a one-CTA shape that would be the
+ * quickest for more than about 100 slices, 19.3 us per iteration of up to 152
+ * against 25.2; its bits differ, so it is by option and autotuner only.)
+ * cluster_sizes[k], resident[k] (n of them): the clusters of each size the
  * device holds at once (0 for a size not listed).  *cluster_size, *clusters receive the choice.
  * Host only.  Errors: PCS_EINVAL, PCS_EUNSUPPORTED (no shape of the size is chosen this way).
  */
@@ -295,7 +303,8 @@ PCS_API pcs_status pcs_solve_slices_f64(const double *field, const unsigned char
  * s0, s1: device complex float32, interleaved (re, im), n_voxels each, 16-byte
  * aligned.  field_out, weight_out: device float32 [n_voxels], 8-byte aligned;
  * mask_out: device uint8 [n_voxels], 2-byte aligned.  Asynchronous on
- * cuda_stream, without any allocation (field_out holds per-CTA maxima meanwhile).  Errors: PCS_EINVAL (NULL, misaligned, t_shift or b0 <= 0,
+ * cuda_stream, without any allocation (field_out holds per-CTA maxima
+ * meanwhile).  Errors: PCS_EINVAL (NULL, misaligned, t_shift or b0 <= 0,
  * threshold < 0), PCS_ECUDA.  n_voxels = 0 is a no-op.
  */
 PCS_API pcs_status pcs_field_map(const float *s0, const float *s1, size_t n_voxels, double t_shift_s,
@@ -398,8 +407,8 @@ typedef struct pcs_tuning {
  * fused primal-dual kernels -- one persistent launch per slice size, run one
  * size after another (the most work first; each launch balances its slices
  * over every resident cluster), with the packing of every size's inputs
- * forked onto per-size streams and everything joined back into cuda_stream.  Step sizes are tau = sigma = 1/L(H, W), L the norm
- * of the full-mask operator K (Sec. II.A pseudocode step 1), computed once per
+ * forked onto per-size streams and everything joined back into cuda_stream.
+ * Step sizes are tau = sigma = 1/L(H, W), L the norm of the full-mask operator K (Sec. II.A pseudocode step 1), computed once per
  * size on the GPU.  autotune != 0: the first solve of a new slice size times
  * every compiled kernel variant of that size on that call's slice count
  * (a short trial) and keeps the fastest -- for calls of other counts too,

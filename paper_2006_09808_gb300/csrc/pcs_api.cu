@@ -132,7 +132,9 @@ static int usable_clusters(const KernelEntry& e, bool smallest, int resident, in
 template <class F>
 static const KernelEntry* cheapest_entry(int H, int W, int is_resident, const ShapeCall& call, int sms, F resident,
                                          int* max_clusters) {
-    auto candidate = [&](const KernelEntry& e) { return e.H == H && e.W == W && e.resident == is_resident && e.us > 0.f; };
+    auto candidate = [&](const KernelEntry& e) {
+        return e.H == H && e.W == W && e.resident == is_resident && e.us > 0.f;
+    };
     int least_C = 0;
     for (const auto& e : entries())
         if (candidate(e) && (least_C == 0 || e.C < least_C) && resident(e) >= 1) least_C = e.C;
@@ -1343,7 +1345,7 @@ pcs_status pcs_batch_tuning(pcs_batch* b, int H, int W, pcs_tuning* out) {
             out->W = W;
             out->L = c.L;
             // the variant of the size's last solve
-            const pcs::KernelEntry* e = c.ctx ? (c.ctx->ran_entry ? c.ctx->ran_entry : c.ctx->entry) : find_entry(H, W, 0);
+            const pcs::KernelEntry* e = !c.ctx ? find_entry(H, W, 0) : c.ctx->ran_entry ? c.ctx->ran_entry : c.ctx->entry;
             out->cluster_size = e ? e->C : 0;
             out->kernel = e ? (e->resident ? 2 : 1) : 0;
             out->threads = e ? e->threads : 0;

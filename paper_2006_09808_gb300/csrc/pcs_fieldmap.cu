@@ -16,8 +16,8 @@
 // map is a programmatic dependent launch.  The
 // maxima lie in the first voxels of field_out, which the map leaves to a third,
 // one-CTA launch: no scratch is allocated (a stream-ordered allocation cost a
-// call that is waited for about 200 us).  256 x 256 x 64 voxels: 29.1 us a call
-// among others (3.6 TB/s of the 25 bytes a voxel needs), 55 us alone; 35.2 and
+// call that is waited for about 200 us).  256 x 256 x 64 voxels: 29-31 us a call
+// among others (3.4-3.6 TB/s of the 25 bytes a voxel needs), 55-60 us alone; 35.2 and
 // 235 before.
 #include <cuda_runtime.h>
 

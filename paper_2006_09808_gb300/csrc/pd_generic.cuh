@@ -313,10 +313,12 @@ __device__ float2* warp_dft(float2* a, float2* b, const float2* T, const GenPlan
                     prime_outputs<2, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, g0, jg, sg);
                 } else if (per % 3 == 0 || per == 5) {
 #pragma unroll 1
-                    for (int j = g0; j < R; j += 3 * jg) prime_outputs<3, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, j, jg, sg);
+                    for (int j = g0; j < R; j += 3 * jg)
+                        prime_outputs<3, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, j, jg, sg);
                 } else {
 #pragma unroll 1
-                    for (int j = g0; j < R; j += 4 * jg) prime_outputs<4, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, j, jg, sg);
+                    for (int j = g0; j < R; j += 4 * jg)
+                        prime_outputs<4, U, A16>(sd, v0, a, P, r, R, Ns, invNs, qp, j, jg, sg);
                 }
             }
             lanes_sync<LP>(id);

@@ -11,8 +11,10 @@
 //     out(k) = D(k) Z(k) - i (2 tau / s) D(k)^2 P(k),     F^-1 out = s v + i u.
 // b is formed from the stored chi in every iteration (nothing is accumulated in the spectrum).  The
 // power of two s ~ 1/lambda (pair_scale) brings W p to the size of b: the rounding that leaks
-// between the channels then stays below that of the separate transforms (measured against FP64
-// over lambda = 1e-5 .. 100).
+// between the channels then stays below that of the separate transforms.  Against FP64, 300 iterations
+// of 64 x 64 emulated in FP32: the same error as with separate transforms for lambda up to 1e-2 (2.5e-7
+// at 5e-4), 5e-7 instead of 1.5e-7 from lambda = 1 on, whatever the scale: u is the transform of chibar
+// before its rounding, which reaches the data term one iteration later.
 //
 // One iteration of a cluster of C CTAs (CTA c owns rows [cR, (c+1)R); column kx is kept together
 // with column W - kx, as the pair of the product above):
@@ -25,10 +27,11 @@
 //
 // A group of T lanes carries rows a = 2j, b = 2j + 1 of the slice for the whole solve, so every thread
 // owns the same 2E pixels throughout and their chi, p, qx, qy never leave the SM: in tensor memory
-// (StTmem: 512 threads x 8E words, 256 KB for E = 16; more than half of the SM's shared memory each,
-// so no two of these CTAs share an SM and the allocation never waits for a peer) or, for small CTAs, in shared memory (StShared).  Neighbouring
-// rows of other groups pass through one row slot per group boundary, which carries chibar of the
-// lower group's row a up and then q_y of the upper group's row b down.
+// (StTmem: 512 threads x 8E words, 256 KB for E = 16; these CTAs take more than half of the SM's
+// shared memory each, so no two of them share an SM and the allocation never waits for a peer) or, for
+// small CTAs, in shared memory (StShared).  Neighbouring rows of other groups pass through one row
+// slot per group boundary, which carries chibar of the lower group's row a up and then q_y of the
+// upper group's row b down.
 //
 // Both rows (in the column pass both columns of a pair) go through every transform together, one in
 // each half of 64-bit registers (F2): one packed instruction for both, half the issue slots.
@@ -39,12 +42,13 @@
 // one CTA, and the strided accesses of the column pass spread over the banks.
 //
 // What bounds it (256 x 256, 4 CTAs of 512 threads): 64 slices x 500 iterations take 19.9 ms, 31.1
-// for pd_cluster.cuh's kernel in the same geometry.  On the way there: scalar transforms of one row after the other, state in tensor memory 35.9 ms (280 bytes of
-// spills, whose reloads miss the small L1); both rows packed 26.0; whole lines per gather instead of
-// 32-byte sectors (column-major units) 21.8; barriers split around independent work, D(k) in flight
-// during one, the field in thread order 19.9.  What is left is the exchange through distributed
-// shared memory (gather, scatter and the barrier behind it, a quarter of an iteration), packed FP32
-// issue (a third), the shared-memory wavefronts of the column pass and the skew at the barriers.
+// for pd_cluster.cuh's kernel in the same geometry.  On the way there: scalar transforms of one row
+// after the other, state in tensor memory 35.9 ms (280 bytes of spills, whose reloads miss the small
+// L1); both rows packed f32x2 26.0; whole lines per gather instead of 32-byte sectors (column-major
+// units) 21.8; barriers split around independent work, D(k) in flight during one, the field in thread
+// order 19.9.  What is left is the exchange through distributed shared memory (gather, scatter and the
+// barrier behind it, a quarter of an iteration), packed FP32 issue (a third), the shared-memory
+// wavefronts of the column pass and the skew at the barriers.
 #pragma once
 
 #include <type_traits>
@@ -72,7 +76,8 @@ struct GeoPair {
     // bytes
     static constexpr size_t SPEC_BYTES = sizeof(float2) * 2 * PC * N;
     static constexpr size_t ROWS_BYTES = sizeof(float2) * NG * N;
-    static constexpr size_t SLOT_BYTES = sizeof(float) * (NG + 1) * N;  // the last one is written by the slice's last rows, read by none
+    // (the last slot is written by the slice's last rows and read by none)
+    static constexpr size_t SLOT_BYTES = sizeof(float) * (NG + 1) * N;
     static constexpr size_t STATE_BYTES = TMEM ? 0 : sizeof(float) * 4 * 2 * E * NT;
     // row slots in shared memory where they fit, else in the chibar scratch rows (global)
     static constexpr size_t BASE_BYTES = SPEC_BYTES + ROWS_BYTES + sizeof(float2) * TW + STATE_BYTES + 16;
