@@ -1,5 +1,7 @@
 """Contexts on streams of their own: the shape follows what else is in flight, the results do not."""
 
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 
@@ -14,7 +16,7 @@ STEP = 1.0 / np.sqrt(4.0 / 9.0 + 8.0)
 
 def problem(H, S, seed):
     pb = phantoms.volume(H, H, S, seed=seed, lam=5e-4, n_iter=40)
-    return torch.from_numpy(pb.field).cuda(), torch.from_numpy(pb.mask).cuda()
+    return torch.from_numpy(pb.field.copy()).cuda(), torch.from_numpy(pb.mask.copy()).cuda()
 
 
 class Call:
@@ -94,3 +96,26 @@ def test_capture_by_the_caller_beside_other_solves():
     assert np.array_equal(ref, one.chi.cpu().numpy())
     volume.close()
     one.close()
+
+
+def test_solves_beside_another_threads_capture():
+    """While this thread captures a graph of its own (global mode), another thread's solves look at what is
+    in flight: they run, and the capture is not invalidated."""
+    st = [torch.cuda.Stream() for _ in range(3)]
+    volume, one = Call(256, 64, 2, 2000, st[0]), Call(256, 1, 1, 40, st[1])
+    x = torch.zeros(64, device="cuda")
+    volume.run()
+    one.run()
+    torch.cuda.synchronize()
+    ref = volume.chi.cpu().numpy(), one.chi.cpu().numpy()
+    g = torch.cuda.CUDAGraph()
+    with ThreadPoolExecutor(1) as ex:
+        with torch.cuda.graph(g, stream=st[2], capture_error_mode="global"):
+            x.add_(1.0)
+            assert ex.submit(lambda: (volume.run(), one.run())).result() == (4, 4)
+            x.add_(1.0)
+    torch.cuda.synchronize()
+    g.replay()
+    torch.cuda.synchronize()
+    assert x.cpu().tolist() == [2.0] * 64
+    assert np.array_equal(ref[0], volume.close()) and np.array_equal(ref[1], one.close())
