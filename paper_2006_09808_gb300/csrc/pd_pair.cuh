@@ -479,7 +479,7 @@ struct StTmem {
         return base + (unsigned)(2 * G::E * a + 4 * c.q);
     }
     // the four arrays' chunk q, in the order q_x, q_y, chi, p.  with_p false: p is not used, and not read
-    // from global memory (chi of the last iteration is being written over it)
+    // from global memory
     __device__ __forceinline__ void load_all(float4 (&v)[4], int q, bool with_p = true) const {
         if constexpr (G::P_GLOBAL) {
             v[3] = with_p ? __ldcg(gp + q * G::NT) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -792,10 +792,15 @@ __device__ __forceinline__ float bit_sel(unsigned bits, int e, float v) { return
 
 // Iterations [it_b, it_e) of slice s: a zero start when it_b = 0 (and no resume), else a
 // continuation from the stored state: chi_{n-1} (in the chibar scratch), p_n, q_n.
-template <class G>
+// P_GLOBAL: in the last pass chi goes where other threads' p lies.  Plain launches load p as ever and store
+// chi after a CTA barrier; scheduled ones do not load it.  Each way is the one that costs its kernel
+// nothing (15 slices of 384 x 384, us per iteration: 48.5 with the two racing on values that nobody uses,
+// 48.3 and 49.4 the two ways; 32 slices, isotropic, on the schedule: 113.7, 114.7 and 113.8).
+template <class G, bool SCHED>
 __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& prm, int s, int it_b, int it_e) {
     constexpr int N = G::N, T = G::T, E = G::E, NCH = G::NCH, C = G::C;
     constexpr unsigned gm = 0xffffffffu;  // the groups of a warp run in step
+    constexpr bool CHI_LATE = G::P_GLOBAL && !SCHED;
     const int lane = threadIdx.x & 31;
     const int grp = threadIdx.x / T;
     const int g = lane % T;
@@ -907,7 +912,7 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
 #pragma unroll
                     for (int q = 0; q < NCH; ++q) {
                         float4 v[4];
-                        cx.st.load_all(v, q, !last);
+                        cx.st.load_all(v, q, CHI_LATE || !last);
                         const float2 qu = G::SLOT_GLOBAL ? u0 : slot.ld_up(q);  // q_y of the row above row a
                         u0 = u1;
                         if (G::SLOT_GLOBAL && q + 2 < NCH) u1 = slot.ld_up(q + 2);
@@ -947,12 +952,21 @@ __device__ __forceinline__ void pair_run_slice(PairCtx<G>& cx, const PDParams& p
                             cx.st.st(kChi, q, make_float4(cn[0].lo(), cn[0].hi(), cn[1].lo(), cn[1].hi()));
                             cx.st.st(kP, q, make_float4(pn[0].lo(), pn[0].hi(), pn[1].lo(), pn[1].hi()));
                             slot.st_up(q, slot_v);
-                        } else {
+                        } else if (!CHI_LATE) {
                             float* o = prm.chi + row0 + T * 2 * q;
                             __stcg(o, cn[0].lo());
                             __stcg(o + N, cn[0].hi());
                             __stcg(o + T, cn[1].lo());
                             __stcg(o + T + N, cn[1].hi());
+                        }
+                        if (CHI_LATE) x[2 * q].y = cn[0], x[2 * q + 1].y = cn[1];  // u is used up
+                    }
+                    if (CHI_LATE && last) {
+                        __syncthreads();  // every thread has loaded its p
+#pragma unroll
+                        for (int e = 0; e < E; ++e) {
+                            __stcg(prm.chi + row0 + T * e, x[e].y.lo());
+                            __stcg(prm.chi + row0 + T * e + N, x[e].y.hi());
                         }
                     }
                 }
@@ -1128,7 +1142,7 @@ __global__ void __launch_bounds__(G::NT, G::MINB) pd_pair_kernel(PDParams prm) {
 #pragma unroll 1
         for (int s = cid; s < prm.S; s += gridDim.x / G::C) {
             if (prm.active && __ldg(prm.active + s) == 0) continue;  // same decision in every CTA of the cluster
-            pair_run_slice<G>(cx, prm, s, 0, prm.n_iter);
+            pair_run_slice<G, false>(cx, prm, s, 0, prm.n_iter);
         }
     } else {
 #pragma unroll 1
@@ -1154,7 +1168,7 @@ __global__ void __launch_bounds__(G::NT, G::MINB) pd_pair_kernel(PDParams prm) {
                 if (threadIdx.x == 0) (void)wait_flag(prm.seg_flags + sg.x, prm.wait_limit);  // this CTA's acquire
                 __syncthreads();
             }
-            pair_run_slice<G>(cx, prm, sg.x, sg.y, sg.z);
+            pair_run_slice<G, true>(cx, prm, sg.x, sg.y, sg.z);
             const int4 done = __ldg(prm.sched + k);
             if (done.w & 2) {
                 cluster_barrier<G::C>();  // every CTA's state is written
